@@ -2,7 +2,10 @@
 // arXiv 2501.06838, Eq. 4 with the Algorithm-1 window): the forward. (The
 // adjoint, one lane per Gaussian over a tile's pixels, is gs_adjoint_tile.cu.)
 //
-// One CTA of NT = TILE*TILE/BY threads renders one TILE x TILE tile of HR
+// Tile 16, one warp per tile: k_raster_fwd16 (the tile in four strips, below);
+// one warp per pair of tiles: k_raster_fwd_pair. The rest of this comment is
+// the layout of tiles 8 and 32, k_raster_fwd:
+// one CTA of NT = TILE*TILE/BY threads renders one TILE x TILE tile of HR
 // pixels; thread t owns column t % TILE and the BY consecutive rows
 // [(t / TILE) * BY, + BY). The tile's Gaussians (a contiguous run of the sorted
 // pair list) go through shared memory in batches of NT * PF, double buffered:
@@ -257,6 +260,284 @@ __device__ __forceinline__ void fwd_gaussian(float2 (&acc)[NQ][3], const FwdOps<
     acc[j][0] = __ffma2_rn(c0, wv, acc[j][0]);
     acc[j][1] = __ffma2_rn(c1, wv, acc[j][1]);
     acc[j][2] = __ffma2_rn(c2, wv, acc[j][2]);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Forward of a 16 x 16 tile by one warp, in four strips of 4 columns x 16 rows.
+//
+// Lane l works on strip l / 8 and owns that strip's four columns on the row
+// pair l % 8 (8 pixels). The strips walk a staged batch independently: a
+// 32-bit mask per strip says which of the batch's Gaussians have a window that
+// meets the strip's columns, and in each step every strip takes its own next
+// one, so a Gaussian costs the strips it touches and not the whole tile.
+// Staging (one lane per Gaussian) leaves everything a step reads as three
+// 16-byte loads: the strip's four column terms Xs = sA (x - cx) (+inf outside
+// the window), the row pair's (-K, -K', R, R') (R = -inf outside the window)
+// and the colour. The slots run backwards (the batch's first Gaussian in the
+// last slot), so that "highest set bit first" is ascending id order and every
+// pixel sums its Gaussians in the order, and with the arithmetic, of the other
+// layouts: the same bits.
+//
+// What bounds it: a 16-byte shared load takes 2.5 cycles of the SM for 1 to 8
+// distinct addresses (4.0 for 32), an FFMA2 2.3 of its scheduler, a MUFU 4.2;
+// the former layout (lane: one column of eight rows) spent 6 such loads, 59
+// scheduler cycles, on 8 pixels per lane whose arithmetic takes 47. Here the
+// step's 3 loads take 36, and the step alone in a loop 64 cycles. Measured
+// against it: 41.2 -> 34.4 us on 65,536 Gaussians at 1024 x 1024 (windows of
+// 22 px on average: 0.68 of the tile's columns per Gaussian), 81.8 -> 53.5 us
+// on 220,052 at 1002 x 751 (14 px), 4134 -> 3776 us on 518,400 at 720 x 720
+// under the ratio window (144 px).
+// ---------------------------------------------------------------------------
+constexpr int kStripSlots = 33;   // 32 slots and, in front, one that adds nothing (odd: no bank conflicts)
+
+template <int PF>
+struct StripTables {
+  float4 x[PF][4 * kStripSlots];   // [strip][slot] Xs of the strip's four columns
+  float4 r[PF][8 * kStripSlots];   // [row pair][slot] (-K(2p), -K(2p+1), R(2p), R(2p+1))
+  float4 c[PF][kStripSlots];       // [slot] colour
+};
+
+// Operands of one step for one lane.
+struct StripOps {
+  float4 x, r, c;
+};
+
+__device__ __forceinline__ void strip_step(float2 (&acc)[2][2][3], const StripOps& o) {
+  const float2 c0 = f2(o.c.x, o.c.x), c1 = f2(o.c.y, o.c.y), c2 = f2(o.c.z, o.c.z);
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {     // the row of the pair
+    const float2 nK = j ? f2(o.r.y, o.r.y) : f2(o.r.x, o.r.x);
+    const float2 R = j ? f2(o.r.w, o.r.w) : f2(o.r.z, o.r.z);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // the columns two by two
+      const float2 d = __fadd2_rn(h ? f2(o.x.z, o.x.w) : f2(o.x.x, o.x.y), nK);
+      const float2 e = __ffma2_rn(f2(-d.x, -d.y), d, R);
+      const float2 wv = f2(ex2_approx(e.x), ex2_approx(e.y));
+      acc[j][h][0] = __ffma2_rn(c0, wv, acc[j][h][0]);
+      acc[j][h][1] = __ffma2_rn(c1, wv, acc[j][h][1]);
+      acc[j][h][2] = __ffma2_rn(c2, wv, acc[j][h][2]);
+    }
+  }
+}
+
+// Stages slot `lane` of one 32-slot table from the Gaussian's record (a lane
+// without a Gaussian: live false) and returns the strips its window meets as
+// four bits.
+__device__ __forceinline__ uint32_t stage_strips(const float4* raw, int lane, bool live, int ox,
+                                                 int oy, float4* tx, float4* tr, float4* tc) {
+  if (!live) return 0u;
+  const float4 f0 = raw[lane], f1 = raw[32 + lane], f2v = raw[64 + lane], f3 = raw[96 + lane];
+  const float cxl = __fadd_rn(__fsub_rn(f0.x, (float)ox), f0.y);
+  const float cyl = __fadd_rn(__fsub_rn(f0.z, (float)oy), f0.w);
+  const int lx0 = __float_as_int(f3.x) - ox, lx1 = __float_as_int(f3.y) - ox;
+  const int ly0 = __float_as_int(f3.z) - oy, ly1 = __float_as_int(f3.w) - oy;
+  uint32_t hit = 0u;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = 4 * q + k;
+      v[k] = f1.x * ((float)c - cxl);
+      if (c < lx0 || c > lx1) v[k] = kInf;
+    }
+    tx[q * kStripSlots + 1 + lane] = make_float4(v[0], v[1], v[2], v[3]);
+    hit |= (lx0 <= 4 * q + 3 && lx1 >= 4 * q) ? 1u << q : 0u;
+  }
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const int r0 = 2 * p, r1 = 2 * p + 1;
+    const float Y0 = (float)r0 - cyl, Y1 = (float)r1 - cyl;
+    float R0 = fmaf(f1.z * Y0, Y0, f1.w), R1 = fmaf(f1.z * Y1, Y1, f1.w);
+    if (r0 < ly0 || r0 > ly1) R0 = -kInf;
+    if (r1 < ly0 || r1 > ly1) R1 = -kInf;
+    tr[p * kStripSlots + 1 + lane] = make_float4(-f1.y * Y0, -f1.y * Y1, R0, R1);
+  }
+  tc[1 + lane] = f2v;
+  return hit;
+}
+
+// The strips' walk over one staged table; m: this lane's strip's mask.
+__device__ __forceinline__ void walk_strips(float2 (&acc)[2][2][3], uint32_t m, int steps,
+                                            const float4* tx, const float4* tr, const float4* tc) {
+  auto load = [&](StripOps& o) {
+    // highest set bit (none: -1, the front slot); the shift of -1 gives 0
+    int b;
+    uint32_t bit;
+    asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(m));
+    asm("shl.b32 %0, 1, %1;" : "=r"(bit) : "r"(b));
+    m ^= bit;
+    o.x = tx[b + 1];
+    o.r = tr[b + 1];
+    o.c = tc[b + 1];
+  };
+  // two operand sets: a step's loads overlap the step before it
+  StripOps A, B;
+  load(A);
+  for (int i = 0; i < steps; i += 2) {
+    load(B);
+    strip_step(acc, A);
+    load(A);
+    strip_step(acc, B);   // past the last step: the front slot, which adds nothing
+  }
+}
+
+template <int PF, bool GRID>
+__global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals) {
+  griddep_release();
+  griddep_wait();
+  constexpr int BATCH = 32 * PF;
+  __shared__ __align__(16) float4 raw[PF][4 * 32];
+  __shared__ StripTables<PF> T;
+  __shared__ uint32_t qbuf[GRID ? GridSource<32, PF>::QCAP : 1];
+
+  const int lane = threadIdx.x;
+  const ImageDesc* D;
+  int ox, oy;
+  tile_origin<16>(w, blockIdx.x, D, ox, oy);
+  const int strip = lane >> 3, rp = lane & 7;
+
+  float2 acc[2][2][3];
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) acc[j][h][0] = acc[j][h][1] = acc[j][h][2] = f2(0.0f, 0.0f);
+  // the front slots: Xs = 0, K = 0, R = -inf, colour 0
+#pragma unroll
+  for (int j = 0; j < PF; ++j) {
+    if (lane < 4) T.x[j][lane * kStripSlots] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane < 8) T.r[j][lane * kStripSlots] = make_float4(0.f, 0.f, -kInf, -kInf);
+    if (lane == 0) T.c[j][0] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+
+  typename std::conditional<GRID, GridSource<32, PF>, SortedSource<32, PF>>::type src;
+  // grid mode: the tile's slice [lbase, lbase + lcount) of the pair list, where
+  // the forward leaves its Gaussian ids (ascending) for the adjoint
+  int lbase = 0, lcount = 0, lpos = 0;
+  bool lok = false;
+  if constexpr (GRID) {
+    grid_source_init<16, 32, PF>(w, D, ox, oy, qbuf, src);
+    {
+      // the tile's pair count: the prefix, along its tile row, of the
+      // footprint pass's per-row differences
+      const int lt = blockIdx.x - D->t_base;
+      const int tyl = lt / D->tiles_x, txl = lt - tyl * D->tiles_x;
+      const uint32_t* row = w.tcount + D->t_base + (int64_t)tyl * D->tiles_x;
+      uint32_t s = 0u;
+      for (int x = lane; x <= txl; x += 32) s += row[x];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      lcount = (int)s;
+    }
+    if (lane == 0) {
+      const unsigned long long b = atomicAdd(&w.hdr->list_cursor, (unsigned long long)lcount);
+      const bool fits = b + (unsigned long long)lcount <= (unsigned long long)w.capacity;
+      lbase = fits ? (int)b : -1;
+      w.ranges[blockIdx.x] = fits ? make_uint2((uint32_t)b, (uint32_t)(b + lcount)) : make_uint2(0u, 0u);
+      if (!fits && lcount > 0) atomicOr(&w.hdr->status, kStCapacity);
+    }
+    lbase = __shfl_sync(0xffffffffu, lbase, 0);
+    lok = lbase >= 0;
+  } else {
+    const uint2 range = w.ranges[blockIdx.x];
+    src.vals = vals;
+    src.pos = (int)range.x;
+    src.end = (int)range.y;
+  }
+  // grid mode: append a batch of ids to the tile's slice of the list
+  auto keep = [&](const uint32_t (&ids)[PF], int n) {
+    if constexpr (GRID) {
+      if (lpos + n > lcount) {   // the footprint count and the tile test disagree
+        if (lane == 0) atomicOr(&w.hdr->status, kStInternal);
+        lok = false;
+      }
+      if (lok) {
+#pragma unroll
+        for (int j = 0; j < PF; ++j) {
+          const int i = j * 32 + lane;
+          if (i < n) w.vals[0][lbase + lpos + i] = ids[j];
+        }
+      }
+      lpos += n;
+    }
+  };
+  // copy a batch's records: entry j * 32 + k goes to table j, slot 31 - k
+  auto issue = [&](const uint32_t (&ids)[PF], int n) {
+#pragma unroll
+    for (int j = 0; j < PF; ++j) {
+      if (j * 32 + lane < n) {
+        const float4* rec = w.records + (int64_t)ids[j] * kRecordF4;
+#pragma unroll
+        for (int q = 0; q < kRecordF4; ++q) cp_async16(&raw[j][q * 32 + 31 - lane], rec + q);
+      }
+    }
+    cp_async_commit();
+  };
+  // batches of the tile's `total` Gaussians (grid mode: the footprint count)
+  int total;
+  if constexpr (GRID) total = lcount; else total = src.end - src.pos;
+  const int nbat = (total + BATCH - 1) / BATCH;
+  uint32_t gid[PF];
+  if (nbat > 0) {
+    keep(gid, src.next(gid));                              // batch 0
+    issue(gid, min(BATCH, total));
+    if (nbat > 1) keep(gid, src.next(gid));                // batch 1
+  }
+  for (int b = 0; b < nbat; ++b) {
+    const int nb = min(BATCH, total - b * BATCH);
+    cp_async_wait_all();
+    __syncwarp();
+    uint32_t m[PF];
+    int steps[PF];
+#pragma unroll
+    for (int j = 0; j < PF; ++j) {
+      const uint32_t hit = stage_strips(raw[j], lane, j * 32 + 31 - lane < nb, ox, oy, T.x[j],
+                                        T.r[j], T.c[j]);
+      m[j] = 0u;
+      steps[j] = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t bal = __ballot_sync(0xffffffffu, (hit >> q) & 1u);
+        steps[j] = max(steps[j], __popc(bal));
+        if (strip == q) m[j] = bal;
+      }
+    }
+    __syncwarp();
+    if (b + 1 < nbat) {
+      issue(gid, min(BATCH, total - (b + 1) * BATCH));
+      if (b + 2 < nbat) keep(gid, src.next(gid));          // batch b + 2
+    }
+#pragma unroll
+    for (int j = 0; j < PF; ++j)
+      walk_strips(acc, m[j], steps[j], T.x[j] + strip * kStripSlots, T.r[j] + rp * kStripSlots,
+                  T.c[j]);
+    __syncwarp();
+  }
+
+  const int H = D->out_h, W = D->out_w;
+  const int x = ox + 4 * strip;
+  float* out = D->out;
+  const int64_t plane = (int64_t)H * W;
+  // four columns per store where the output's rows are 16-byte aligned
+  const bool vec = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int y = oy - D->row0 + 2 * rp + j;   // output row
+    if (y >= H || x >= W) continue;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      float* o = out + k * plane + (int64_t)y * W + x;
+      const float2 a = acc[j][0][k], b = acc[j][1][k];
+      if (vec) {
+        *reinterpret_cast<float4*>(o) = make_float4(a.x, a.y, b.x, b.y);
+      } else {
+        o[0] = a.x;
+        if (x + 1 < W) o[1] = a.y;
+        if (x + 2 < W) o[2] = b.x;
+        if (x + 3 < W) o[3] = b.y;
+      }
+    }
   }
 }
 
@@ -743,6 +1024,13 @@ cudaError_t run(const Ws& w, const uint32_t* vals, cudaStream_t s) {
   return launch_chain(k_raster_fwd<TILE, BY, PF, false>, dim3(w.tiles), dim3(NT), 0, s, w, vals);
 }
 
+template <int PF>
+cudaError_t run16(const Ws& w, const uint32_t* vals, cudaStream_t s) {
+  LaunchScope ls(kKRasterFwd, s);
+  if (w.grid) return launch_chain(k_raster_fwd16<PF, true>, dim3(w.tiles), dim3(32), 0, s, w, vals);
+  return launch_chain(k_raster_fwd16<PF, false>, dim3(w.tiles), dim3(32), 0, s, w, vals);
+}
+
 // Launch configurations: tile edge -> rows per thread (threads = TILE^2 / BY);
 // batch = Gaussians staged per round = threads * PF, PF in {1, 2} (the host
 // accepts only these batches; 0 selects PF = 1).
@@ -760,7 +1048,7 @@ cudaError_t dispatch(const Ws& w, const uint32_t* vals, int batch, cudaStream_t 
     case 32:  // 64 threads
       return batch >= 128 ? run<32, 16, 2>(w, vals, s) : run<32, 16, 1>(w, vals, s);
     default:  // 32 threads
-      return batch >= 64 ? run<16, 8, 2>(w, vals, s) : run<16, 8, 1>(w, vals, s);
+      return batch >= 64 ? run16<2>(w, vals, s) : run16<1>(w, vals, s);
   }
 }
 
