@@ -140,11 +140,10 @@ typedef enum { GS_BINNING_AUTO = 0, GS_BINNING_SORT = 1, GS_BINNING_GRID = 2 } g
  * parameter: the image is the same bit for bit):
  *   TILE: one warp per tile (tile 16: four strips of 4 columns, each walking
  *         the Gaussians whose window meets it);
- *   PAIR: one warp per horizontal pair of 16 x 16 tiles, each thread one
- *         column of each tile: the per-Gaussian work (shared-memory staging,
- *         operand loads) is shared by the two tiles, and each tile is computed
- *         only for the Gaussians whose window meets it. Needs GRID binning and
- *         tile 16 (GS_ERR_UNSUPPORTED otherwise);
+ *   PAIR: one warp per horizontal pair of 16 x 16 tiles, in four strips of 8
+ *         columns: the per-Gaussian work (shared-memory staging, operand
+ *         loads) is shared by the two tiles. Needs GRID binning and tile 16
+ *         (GS_ERR_UNSUPPORTED otherwise);
  *   AUTO: PAIR with GRID binning at tile 16 when every view uses the SIGMA
  *         window and some view's scale is >= 6 (large windows, where it
  *         measured faster), else TILE. */

@@ -291,27 +291,42 @@ __device__ __forceinline__ void fwd_gaussian(float2 (&acc)[NQ][3], const FwdOps<
 // ---------------------------------------------------------------------------
 constexpr int kStripSlots = 33;   // 32 slots and, in front, one that adds nothing (odd: no bank conflicts)
 
-template <int PF>
+// NQ: groups of four columns per strip and lane (1: the strips of one tile; 2:
+// strips of 8 columns over a pair of tiles).
+template <int NQ>
 struct StripTables {
-  float4 x[PF][4 * kStripSlots];   // [strip][slot] Xs of the strip's four columns
-  float4 r[PF][8 * kStripSlots];   // [row pair][slot] (-K(2p), -K(2p+1), R(2p), R(2p+1))
-  float4 c[PF][kStripSlots];       // [slot] colour
+  float4 x[4 * NQ * kStripSlots];   // [strip][quad][slot] Xs of four columns
+  float4 r[8 * kStripSlots];        // [row pair][slot] (-K(2p), -K(2p+1), R(2p), R(2p+1))
+  float4 c[kStripSlots];            // [slot] colour
+  // the front slots: Xs = 0, K = 0, R = -inf, colour 0
+  __device__ __forceinline__ void clear_front(int lane) {
+    if (lane < 4 * NQ) x[lane * kStripSlots] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane < 8) r[lane * kStripSlots] = make_float4(0.f, 0.f, -kInf, -kInf);
+    if (lane == 0) c[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
 };
+
+// A lane's pixels: [row of its pair][column pair][channel].
+template <int NQ>
+using StripAcc = float2[2][2 * NQ][3];
 
 // Operands of one step for one lane.
+template <int NQ>
 struct StripOps {
-  float4 x, r, c;
+  float4 x[NQ], r, c;
 };
 
-__device__ __forceinline__ void strip_step(float2 (&acc)[2][2][3], const StripOps& o) {
+template <int NQ>
+__device__ __forceinline__ void strip_step(StripAcc<NQ>& acc, const StripOps<NQ>& o) {
   const float2 c0 = f2(o.c.x, o.c.x), c1 = f2(o.c.y, o.c.y), c2 = f2(o.c.z, o.c.z);
 #pragma unroll
   for (int j = 0; j < 2; ++j) {     // the row of the pair
     const float2 nK = j ? f2(o.r.y, o.r.y) : f2(o.r.x, o.r.x);
     const float2 R = j ? f2(o.r.w, o.r.w) : f2(o.r.z, o.r.z);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {   // the columns two by two
-      const float2 d = __fadd2_rn(h ? f2(o.x.z, o.x.w) : f2(o.x.x, o.x.y), nK);
+    for (int h = 0; h < 2 * NQ; ++h) {   // the columns two by two
+      const float4 xq = o.x[h / 2];
+      const float2 d = __fadd2_rn((h & 1) ? f2(xq.z, xq.w) : f2(xq.x, xq.y), nK);
       const float2 e = __ffma2_rn(f2(-d.x, -d.y), d, R);
       const float2 wv = f2(ex2_approx(e.x), ex2_approx(e.y));
       acc[j][h][0] = __ffma2_rn(c0, wv, acc[j][h][0]);
@@ -321,30 +336,34 @@ __device__ __forceinline__ void strip_step(float2 (&acc)[2][2][3], const StripOp
   }
 }
 
-// Stages slot `lane` of one 32-slot table from the Gaussian's record (a lane
-// without a Gaussian: live false) and returns the strips its window meets as
-// four bits.
+// Stages slot `lane` of a table from the Gaussian's record (a lane without a
+// Gaussian: live false) and returns the strips its window meets as four bits.
+// Column terms are relative to the 16-column tile they belong to.
+template <int NQ>
 __device__ __forceinline__ uint32_t stage_strips(const float4* raw, int lane, bool live, int ox,
-                                                 int oy, float4* tx, float4* tr, float4* tc) {
+                                                 int oy, StripTables<NQ>& t) {
   if (!live) return 0u;
   const float4 f0 = raw[lane], f1 = raw[32 + lane], f2v = raw[64 + lane], f3 = raw[96 + lane];
-  const float cxl = __fadd_rn(__fsub_rn(f0.x, (float)ox), f0.y);
   const float cyl = __fadd_rn(__fsub_rn(f0.z, (float)oy), f0.w);
   const int lx0 = __float_as_int(f3.x) - ox, lx1 = __float_as_int(f3.y) - ox;
   const int ly0 = __float_as_int(f3.z) - oy, ly1 = __float_as_int(f3.w) - oy;
   uint32_t hit = 0u;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
+  for (int q = 0; q < 4 * NQ; ++q) {
+    const int tx = 16 * (q / 4);   // the tile's first column
+    const float cxl = __fadd_rn(__fsub_rn(f0.x, (float)(ox + tx)), f0.y);
     float v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int c = 4 * q + k;
-      v[k] = f1.x * ((float)c - cxl);
+      v[k] = f1.x * ((float)(c - tx) - cxl);
       if (c < lx0 || c > lx1) v[k] = kInf;
     }
-    tx[q * kStripSlots + 1 + lane] = make_float4(v[0], v[1], v[2], v[3]);
-    hit |= (lx0 <= 4 * q + 3 && lx1 >= 4 * q) ? 1u << q : 0u;
+    t.x[q * kStripSlots + 1 + lane] = make_float4(v[0], v[1], v[2], v[3]);
   }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    hit |= (lx0 <= 4 * NQ * (q + 1) - 1 && lx1 >= 4 * NQ * q) ? 1u << q : 0u;
 #pragma unroll
   for (int p = 0; p < 8; ++p) {
     const int r0 = 2 * p, r1 = 2 * p + 1;
@@ -352,34 +371,104 @@ __device__ __forceinline__ uint32_t stage_strips(const float4* raw, int lane, bo
     float R0 = fmaf(f1.z * Y0, Y0, f1.w), R1 = fmaf(f1.z * Y1, Y1, f1.w);
     if (r0 < ly0 || r0 > ly1) R0 = -kInf;
     if (r1 < ly0 || r1 > ly1) R1 = -kInf;
-    tr[p * kStripSlots + 1 + lane] = make_float4(-f1.y * Y0, -f1.y * Y1, R0, R1);
+    t.r[p * kStripSlots + 1 + lane] = make_float4(-f1.y * Y0, -f1.y * Y1, R0, R1);
   }
-  tc[1 + lane] = f2v;
+  t.c[1 + lane] = f2v;
   return hit;
 }
 
-// The strips' walk over one staged table; m: this lane's strip's mask.
-__device__ __forceinline__ void walk_strips(float2 (&acc)[2][2][3], uint32_t m, int steps,
-                                            const float4* tx, const float4* tr, const float4* tc) {
-  auto load = [&](StripOps& o) {
-    // highest set bit (none: -1, the front slot); the shift of -1 gives 0
+// One staged table: the strips' masks from the lanes' hits, then the walk.
+// Returns nothing; every lane adds its strip's Gaussians to acc.
+struct StripMasks {
+  uint32_t m;   // this lane's strip's mask
+  int steps;    // the largest number of Gaussians any strip has
+};
+__device__ __forceinline__ StripMasks strip_masks(uint32_t hit, int strip) {
+  StripMasks s{0u, 0};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const uint32_t bal = __ballot_sync(0xffffffffu, (hit >> q) & 1u);
+    s.steps = max(s.steps, __popc(bal));
+    if (strip == q) s.m = bal;
+  }
+  return s;
+}
+
+template <int NQ>
+__device__ __forceinline__ void walk_strips(StripAcc<NQ>& acc, StripMasks s, int strip, int rp,
+                                            const StripTables<NQ>& t) {
+  const float4* tx = t.x + strip * NQ * kStripSlots;
+  const float4* tr = t.r + rp * kStripSlots;
+  uint32_t m = s.m;
+  auto load = [&](StripOps<NQ>& o) {
+    // highest set bit (none: -1, the front slot); the shift by -1 gives 0
     int b;
     uint32_t bit;
     asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(m));
     asm("shl.b32 %0, 1, %1;" : "=r"(bit) : "r"(b));
     m ^= bit;
-    o.x = tx[b + 1];
+#pragma unroll
+    for (int h = 0; h < NQ; ++h) o.x[h] = tx[b + 1 + h * kStripSlots];
     o.r = tr[b + 1];
-    o.c = tc[b + 1];
+    o.c = t.c[b + 1];
   };
   // two operand sets: a step's loads overlap the step before it
-  StripOps A, B;
+  StripOps<NQ> A, B;
   load(A);
-  for (int i = 0; i < steps; i += 2) {
+  for (int i = 0; i < s.steps; i += 2) {
     load(B);
-    strip_step(acc, A);
+    strip_step<NQ>(acc, A);
     load(A);
-    strip_step(acc, B);   // past the last step: the front slot, which adds nothing
+    strip_step<NQ>(acc, B);   // past the last step: the front slot, which adds nothing
+  }
+}
+
+// Copies the records of a batch: entry j * 32 + k goes to raw[j], slot 31 - k.
+template <int PF>
+__device__ __forceinline__ void issue_slots(const Ws& w, const uint32_t (&ids)[PF], int n,
+                                            float4 (&raw)[PF][4 * 32]) {
+  const int lane = threadIdx.x;
+#pragma unroll
+  for (int j = 0; j < PF; ++j) {
+    if (j * 32 + lane < n) {
+      const float4* rec = w.records + (int64_t)ids[j] * kRecordF4;
+#pragma unroll
+      for (int q = 0; q < kRecordF4; ++q) cp_async16(&raw[j][q * 32 + 31 - lane], rec + q);
+    }
+  }
+  cp_async_commit();
+}
+
+// Writes a lane's pixels: columns x .., rows y and y + 1 of the output.
+template <int NQ>
+__device__ __forceinline__ void store_strips(const ImageDesc* D, const StripAcc<NQ>& acc, int x,
+                                             int y) {
+  const int H = D->out_h, W = D->out_w;
+  float* out = D->out;
+  const int64_t plane = (int64_t)H * W;
+  // four columns per store where the output's rows are 16-byte aligned
+  const bool vec = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    if (y + j >= H) continue;
+#pragma unroll
+    for (int h = 0; h < NQ; ++h) {
+      const int xh = x + 4 * h;
+      if (xh >= W) continue;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        float* o = out + k * plane + (int64_t)(y + j) * W + xh;
+        const float2 a = acc[j][2 * h][k], b = acc[j][2 * h + 1][k];
+        if (vec) {
+          *reinterpret_cast<float4*>(o) = make_float4(a.x, a.y, b.x, b.y);
+        } else {
+          o[0] = a.x;
+          if (xh + 1 < W) o[1] = a.y;
+          if (xh + 2 < W) o[2] = b.x;
+          if (xh + 3 < W) o[3] = b.y;
+        }
+      }
+    }
   }
 }
 
@@ -389,7 +478,7 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
   griddep_wait();
   constexpr int BATCH = 32 * PF;
   __shared__ __align__(16) float4 raw[PF][4 * 32];
-  __shared__ StripTables<PF> T;
+  __shared__ StripTables<1> T[PF];
   __shared__ uint32_t qbuf[GRID ? GridSource<32, PF>::QCAP : 1];
 
   const int lane = threadIdx.x;
@@ -398,18 +487,13 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
   tile_origin<16>(w, blockIdx.x, D, ox, oy);
   const int strip = lane >> 3, rp = lane & 7;
 
-  float2 acc[2][2][3];
+  StripAcc<1> acc;
 #pragma unroll
   for (int j = 0; j < 2; ++j)
 #pragma unroll
     for (int h = 0; h < 2; ++h) acc[j][h][0] = acc[j][h][1] = acc[j][h][2] = f2(0.0f, 0.0f);
-  // the front slots: Xs = 0, K = 0, R = -inf, colour 0
 #pragma unroll
-  for (int j = 0; j < PF; ++j) {
-    if (lane < 4) T.x[j][lane * kStripSlots] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (lane < 8) T.r[j][lane * kStripSlots] = make_float4(0.f, 0.f, -kInf, -kInf);
-    if (lane == 0) T.c[j][0] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+  for (int j = 0; j < PF; ++j) T[j].clear_front(lane);
 
   typename std::conditional<GRID, GridSource<32, PF>, SortedSource<32, PF>>::type src;
   // grid mode: the tile's slice [lbase, lbase + lcount) of the pair list, where
@@ -462,18 +546,6 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
       lpos += n;
     }
   };
-  // copy a batch's records: entry j * 32 + k goes to table j, slot 31 - k
-  auto issue = [&](const uint32_t (&ids)[PF], int n) {
-#pragma unroll
-    for (int j = 0; j < PF; ++j) {
-      if (j * 32 + lane < n) {
-        const float4* rec = w.records + (int64_t)ids[j] * kRecordF4;
-#pragma unroll
-        for (int q = 0; q < kRecordF4; ++q) cp_async16(&raw[j][q * 32 + 31 - lane], rec + q);
-      }
-    }
-    cp_async_commit();
-  };
   // batches of the tile's `total` Gaussians (grid mode: the footprint count)
   int total;
   if constexpr (GRID) total = lcount; else total = src.end - src.pos;
@@ -481,64 +553,28 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
   uint32_t gid[PF];
   if (nbat > 0) {
     keep(gid, src.next(gid));                              // batch 0
-    issue(gid, min(BATCH, total));
+    issue_slots<PF>(w, gid, min(BATCH, total), raw);
     if (nbat > 1) keep(gid, src.next(gid));                // batch 1
   }
   for (int b = 0; b < nbat; ++b) {
     const int nb = min(BATCH, total - b * BATCH);
     cp_async_wait_all();
     __syncwarp();
-    uint32_t m[PF];
-    int steps[PF];
+    StripMasks ms[PF];
 #pragma unroll
-    for (int j = 0; j < PF; ++j) {
-      const uint32_t hit = stage_strips(raw[j], lane, j * 32 + 31 - lane < nb, ox, oy, T.x[j],
-                                        T.r[j], T.c[j]);
-      m[j] = 0u;
-      steps[j] = 0;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t bal = __ballot_sync(0xffffffffu, (hit >> q) & 1u);
-        steps[j] = max(steps[j], __popc(bal));
-        if (strip == q) m[j] = bal;
-      }
-    }
+    for (int j = 0; j < PF; ++j)
+      ms[j] = strip_masks(stage_strips<1>(raw[j], lane, j * 32 + 31 - lane < nb, ox, oy, T[j]), strip);
     __syncwarp();
     if (b + 1 < nbat) {
-      issue(gid, min(BATCH, total - (b + 1) * BATCH));
+      issue_slots<PF>(w, gid, min(BATCH, total - (b + 1) * BATCH), raw);
       if (b + 2 < nbat) keep(gid, src.next(gid));          // batch b + 2
     }
 #pragma unroll
-    for (int j = 0; j < PF; ++j)
-      walk_strips(acc, m[j], steps[j], T.x[j] + strip * kStripSlots, T.r[j] + rp * kStripSlots,
-                  T.c[j]);
+    for (int j = 0; j < PF; ++j) walk_strips<1>(acc, ms[j], strip, rp, T[j]);
     __syncwarp();
   }
 
-  const int H = D->out_h, W = D->out_w;
-  const int x = ox + 4 * strip;
-  float* out = D->out;
-  const int64_t plane = (int64_t)H * W;
-  // four columns per store where the output's rows are 16-byte aligned
-  const bool vec = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const int y = oy - D->row0 + 2 * rp + j;   // output row
-    if (y >= H || x >= W) continue;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      float* o = out + k * plane + (int64_t)y * W + x;
-      const float2 a = acc[j][0][k], b = acc[j][1][k];
-      if (vec) {
-        *reinterpret_cast<float4*>(o) = make_float4(a.x, a.y, b.x, b.y);
-      } else {
-        o[0] = a.x;
-        if (x + 1 < W) o[1] = a.y;
-        if (x + 2 < W) o[2] = b.x;
-        if (x + 3 < W) o[3] = b.y;
-      }
-    }
-  }
+  store_strips<1>(D, acc, ox + 4 * strip, oy - D->row0 + 2 * rp);
 }
 
 template <int TILE, int BY, int PF, bool GRID>
@@ -673,16 +709,24 @@ __global__ void __launch_bounds__(TILE * TILE / BY) k_raster_fwd(Ws w, const uin
 
 // ---------------------------------------------------------------------------
 // Forward over a pair of horizontally adjacent 16 x 16 tiles (grid-implicit
-// binning, tile 16): one warp renders a 32 x 16 region; lane l owns columns
-// c = l % 16 (tile A) and c + 16 (tile B), rows (l / 16) * 8 .. + 8. The pair's
-// candidates are enumerated once; each kept Gaussian carries whether its
-// window meets tile A, tile B or both, and each half is computed only for the
-// Gaussians that meet it (a warp-uniform test), so the evaluated pixels are
-// those of 16 x 16 tiles while the per-Gaussian work (staging, operand loads,
-// loop) is shared by up to 16 pixels per lane. The two tiles' lists are left
-// for the adjoint exactly as the single-tile forward leaves them (same
-// Gaussians, ascending ids), and every pixel sums its Gaussians in the same
-// order, so the image is bitwise the single-tile forward's.
+// binning, tile 16): one warp renders a 32 x 16 region in four strips of 8
+// columns (two per tile), each lane 8 columns of a row pair, so that a step's
+// loads and mask work serve 16 pixels. The pair's candidates are enumerated and
+// staged once; the two tiles' lists are left for the adjoint exactly as the
+// single-tile forward leaves them (same Gaussians, ascending ids). Column
+// terms are relative to their own tile and every pixel sums its Gaussians in
+// the same order, so the image is bitwise the single-tile forward's.
+//
+// A step in a loop of its own takes 111 scheduler cycles for 16 pixels per
+// lane, the single tile's 64 for 8: the arithmetic (94 at 2.3 cycles per FFMA2)
+// bounds it. Against the former pair layout (each lane a column of both tiles,
+// 7 shared loads per 16 pixels): 1168 -> 1007 us on 518,400 Gaussians at
+// 5760 x 3240 (windows of 74 px on average), 857 -> 799 us on 16 uneven images,
+// 87 -> 73 us at scale 24. Wider strips cost small windows more columns, so
+// scales below 6 keep single tiles (1002 x 751 at scale 3.7, 14 px windows: 52
+// against 70 us). The register cap (128, no spills) gives 16 CTAs per SM; 18
+// CTAs (112, spills) were 2% faster on the uneven batch and 1% to 10% slower
+// elsewhere.
 // ---------------------------------------------------------------------------
 template <int PF>
 struct PairSource {
@@ -744,113 +788,13 @@ struct PairSource {
   }
 };
 
-// Stage 1 for a pair, each half exactly as the single-tile forward stages it
-// for that tile (so the image is bitwise the same):
-//   gA = (cxl_a, sA, lx0_a, lx1_a)   gD = (cxl_b, lx0_b, lx1_b, 0)
-//   gB = (cyl, sK, g, l)             gC = (r, g, b, ly0 | ly1 << 16)
-// with cxl_h the centre relative to half h's first column and [lx0_h, lx1_h]
-// the window's columns in that half (empty when lx0_h > lx1_h).
-template <int NT>
-__device__ __forceinline__ void stage_pair_records(const float4* raw, int nb, int ox, int oy,
-                                                   float4* gA, float4* gB, float4* gC,
-                                                   float4* gD) {
-  for (int i = threadIdx.x; i < nb; i += NT) {
-    const float4 f0 = raw[i * kRecordF4], f1 = raw[i * kRecordF4 + 1];
-    const float4 f2 = raw[i * kRecordF4 + 2], f3 = raw[i * kRecordF4 + 3];
-    const int ob = ox + 16;
-    const float cxa = __fadd_rn(__fsub_rn(f0.x, (float)ox), f0.y);
-    const float cxb = __fadd_rn(__fsub_rn(f0.x, (float)ob), f0.y);
-    const float cyl = __fadd_rn(__fsub_rn(f0.z, (float)oy), f0.w);
-    const int x0 = __float_as_int(f3.x), x1 = __float_as_int(f3.y);
-    const int ly0 = max(__float_as_int(f3.z) - oy, 0), ly1 = min(__float_as_int(f3.w) - oy, 15);
-    gA[i] = make_float4(cxa, f1.x, (float)max(x0 - ox, 0), (float)min(x1 - ox, 15));
-    gD[i] = make_float4(cxb, (float)max(x0 - ob, 0), (float)min(x1 - ob, 15), 0.0f);
-    gB[i] = make_float4(cyl, f1.y, f1.z, f1.w);
-    gC[i] = make_float4(f2.x, f2.y, f2.z, __int_as_float(ly0 | (ly1 << 16)));
-  }
-}
-
-// Operands of one Gaussian for one lane of the pair kernel.
-struct PairOps {
-  float4 a, d, c, q[4];
-  __device__ __forceinline__ void load(const float4* gA, const float4* gD, const float4* gC,
-                                       const float4* rq, int i, int pair0) {
-    a = gA[i];
-    d = gD[i];
-    c = gC[i];
-    const float4* rr = rq + i * 8 + pair0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) q[j] = rr[j];
-  }
-};
-
-// One Gaussian on one 16-column half: centre cxl, window columns [lo, hi].
-__device__ __forceinline__ void fwd_half(float2 (&acc)[4][3], const float4 (&q)[4], float sA,
-                                         float cxl, float lo, float hi, float fcol, float2 c0,
-                                         float2 c1, float2 c2) {
-  float Xs = sA * (fcol - cxl);
-  if (fcol < lo || fcol > hi) Xs = kInf;
-  const float2 X2 = f2(Xs, Xs);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float2 d = __fadd2_rn(X2, f2(q[j].x, q[j].y));
-    const float2 e = __ffma2_rn(f2(-d.x, -d.y), d, f2(q[j].z, q[j].w));
-    const float2 wv = f2(ex2_approx(e.x), ex2_approx(e.y));
-    acc[j][0] = __ffma2_rn(c0, wv, acc[j][0]);
-    acc[j][1] = __ffma2_rn(c1, wv, acc[j][1]);
-    acc[j][2] = __ffma2_rn(c2, wv, acc[j][2]);
-  }
-}
-
-// Both halves at once: the two halves' eight row-pair chains interleave.
-__device__ __forceinline__ void fwd_both(float2 (&accA)[4][3], float2 (&accB)[4][3],
-                                         const PairOps& o, float fcol, float2 c0, float2 c1,
-                                         float2 c2) {
-  float XsA = o.a.y * (fcol - o.a.x);
-  if (fcol < o.a.z || fcol > o.a.w) XsA = kInf;
-  float XsB = o.a.y * (fcol - o.d.x);
-  if (fcol < o.d.y || fcol > o.d.z) XsB = kInf;
-  const float2 XA = f2(XsA, XsA), XB = f2(XsB, XsB);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float2 nK = f2(o.q[j].x, o.q[j].y), R = f2(o.q[j].z, o.q[j].w);
-    const float2 da = __fadd2_rn(XA, nK), db = __fadd2_rn(XB, nK);
-    const float2 ea = __ffma2_rn(f2(-da.x, -da.y), da, R);
-    const float2 eb = __ffma2_rn(f2(-db.x, -db.y), db, R);
-    const float2 wa = f2(ex2_approx(ea.x), ex2_approx(ea.y));
-    const float2 wb = f2(ex2_approx(eb.x), ex2_approx(eb.y));
-    accA[j][0] = __ffma2_rn(c0, wa, accA[j][0]);
-    accB[j][0] = __ffma2_rn(c0, wb, accB[j][0]);
-    accA[j][1] = __ffma2_rn(c1, wa, accA[j][1]);
-    accB[j][1] = __ffma2_rn(c1, wb, accB[j][1]);
-    accA[j][2] = __ffma2_rn(c2, wa, accA[j][2]);
-    accB[j][2] = __ffma2_rn(c2, wb, accB[j][2]);
-  }
-}
-
-__device__ __forceinline__ void fwd_pair_gaussian(float2 (&accA)[4][3], float2 (&accB)[4][3],
-                                                  const PairOps& o, float fcol) {
-  const float2 c0 = f2(o.c.x, o.c.x), c1 = f2(o.c.y, o.c.y), c2 = f2(o.c.z, o.c.z);
-  const bool ha = o.a.z <= o.a.w, hb = o.d.y <= o.d.z;   // meets tile A / B (warp-uniform)
-  if (ha && hb)
-    fwd_both(accA, accB, o, fcol, c0, c1, c2);
-  else if (ha)
-    fwd_half(accA, o.q, o.a.y, o.a.x, o.a.z, o.a.w, fcol, c0, c1, c2);
-  else
-    fwd_half(accB, o.q, o.a.y, o.d.x, o.d.y, o.d.z, fcol, c0, c1, c2);
-}
-
-// PF = 1: 18 resident CTAs per SM (shared memory allows 18); the cap takes it
-// from 110 to 93 registers with no spills. PF = 2 is held to 9 by shared memory.
 template <int PF>
-__global__ void __launch_bounds__(32, PF == 1 ? 18 : 1) k_raster_fwd_pair(Ws w) {
+__global__ void __launch_bounds__(32, 16) k_raster_fwd_pair(Ws w) {
   griddep_release();
   griddep_wait();
-  constexpr int NT = 32, BATCH = NT * PF;
   using Src = PairSource<PF>;
-  __shared__ __align__(16) float4 raw[2][BATCH * kRecordF4];
-  __shared__ float4 gA[BATCH], gB[BATCH], gC[BATCH], gD[BATCH];
-  __shared__ float4 rq[BATCH * 8];
+  __shared__ __align__(16) float4 raw[PF][4 * 32];
+  __shared__ StripTables<2> T[PF];
   __shared__ uint32_t qbuf[Src::QCAP];
   __shared__ uint8_t qflg[Src::QCAP];
   __shared__ int sbase;
@@ -934,7 +878,7 @@ __global__ void __launch_bounds__(32, PF == 1 ? 18 : 1) k_raster_fwd_pair(Ws w) 
   auto keep = [&](const uint32_t (&ids)[PF], const uint32_t (&fl)[PF], int n) {
 #pragma unroll
     for (int j = 0; j < PF; ++j) {
-      const int i = j * NT + lane;
+      const int i = j * 32 + lane;
       const bool fa = i < n && (fl[j] & 1u), fb = i < n && (fl[j] & 2u);
       const unsigned ba = __ballot_sync(0xffffffffu, fa), bb = __ballot_sync(0xffffffffu, fb);
       const unsigned lt = (1u << lane) - 1u;
@@ -950,44 +894,40 @@ __global__ void __launch_bounds__(32, PF == 1 ? 18 : 1) k_raster_fwd_pair(Ws w) 
     }
   };
 
-  const int c = lane & 15;
-  const int pair0 = (lane >> 4) * 4;
-  const float fcol = (float)c;
-  float2 accA[4][3], accB[4][3];
+  const int strip = lane >> 3, rp = lane & 7;
+  StripAcc<2> acc;
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+  for (int j = 0; j < 2; ++j)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) accA[j][k] = accB[j][k] = f2(0.0f, 0.0f);
+    for (int h = 0; h < 4; ++h) acc[j][h][0] = acc[j][h][1] = acc[j][h][2] = f2(0.0f, 0.0f);
+#pragma unroll
+  for (int j = 0; j < PF; ++j) T[j].clear_front(lane);
 
   uint32_t gid[PF], fl[PF];
   int nb0 = src.next(gid, fl);   // batch 0
   keep(gid, fl, nb0);
   int nb1 = 0;
   if (nb0 > 0) {
-    issue_records<NT, PF>(w, gid, nb0, raw[0]);
+    issue_slots<PF>(w, gid, nb0, raw);
     nb1 = src.next(gid, fl);      // batch 1
     keep(gid, fl, nb1);
   }
-  for (int b = 0; nb0 > 0; ++b) {
+  while (nb0 > 0) {
     cp_async_wait_all();
     __syncwarp();
-    stage_pair_records<NT>(raw[b & 1], nb0, ox, oy, gA, gB, gC, gD);
-    __syncwarp();
-    stage_rowpairs<16, NT>(nb0, gB, gC, rq);
+    StripMasks ms[PF];
+#pragma unroll
+    for (int j = 0; j < PF; ++j)
+      ms[j] = strip_masks(stage_strips<2>(raw[j], lane, j * 32 + 31 - lane < nb0, ox, oy, T[j]), strip);
     __syncwarp();
     int nb2 = 0;
     if (nb1 > 0) {
-      issue_records<NT, PF>(w, gid, nb1, raw[(b + 1) & 1]);
+      issue_slots<PF>(w, gid, nb1, raw);
       nb2 = src.next(gid, fl);    // batch b + 2
       keep(gid, fl, nb2);
     }
-    // One operand set in registers (a second one for overlapping the next
-    // Gaussian's loads measured slower: the registers cost more warps)
-    for (int i = 0; i < nb0; ++i) {
-      PairOps A;
-      A.load(gA, gD, gC, rq, i, pair0);
-      fwd_pair_gaussian(accA, accB, A, fcol);
-    }
+#pragma unroll
+    for (int j = 0; j < PF; ++j) walk_strips<2>(acc, ms[j], strip, rp, T[j]);
     __syncwarp();
     nb0 = nb1;
     nb1 = nb2;
@@ -996,24 +936,7 @@ __global__ void __launch_bounds__(32, PF == 1 ? 18 : 1) k_raster_fwd_pair(Ws w) 
     if (lane == 0) atomicOr(&w.hdr->status, kStInternal);
   }
 
-  const int H = D->out_h, W = D->out_w;
-  float* out = D->out;
-  const int64_t plane = (int64_t)H * W;
-  auto store = [&](const float2 (&acc)[4][3], int x) {
-    if (x >= W) return;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int y = oy - D->row0 + pair0 * 2 + k;   // output row
-      if (y < H) {
-        const int64_t o = (int64_t)y * W + x;
-        out[o] = (k & 1) ? acc[k / 2][0].y : acc[k / 2][0].x;
-        out[plane + o] = (k & 1) ? acc[k / 2][1].y : acc[k / 2][1].x;
-        out[2 * plane + o] = (k & 1) ? acc[k / 2][2].y : acc[k / 2][2].x;
-      }
-    }
-  };
-  store(accA, ox + c);
-  store(accB, ox + 16 + c);
+  store_strips<2>(D, acc, ox + 8 * strip, oy - D->row0 + 2 * rp);
 }
 
 template <int TILE, int BY, int PF>
