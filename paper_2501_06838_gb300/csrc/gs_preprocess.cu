@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(kFootprintBlock) k_preprocess(Ws w) {
       // Gaussian's LR cell (i, j): DL = s j - x0, DR = x1 - s j (rows alike),
       // rounded up, plus one pixel of margin for the float32 rounding of s j
       const bool live = x0 <= x1 && y0 <= y1;
-      w.win[gi] = live ? make_short4((short)x0, (short)x1, (short)y0, (short)y1)
-                       : make_short4(32767, -32768, 32767, -32768);
+      w.win[gi] = live ? make_short4((short)x0, (short)y0, (short)x1, (short)y1)
+                       : make_short4(32767, 32767, -32768, -32768);
       if (live) {
         const int64_t cell = li / D.m;
         const float sj = s * (float)(cell % D.lr_w), si = s * (float)(cell / D.lr_w);
