@@ -112,6 +112,7 @@ struct Ws {
   int32_t n_pairs;            // grid binning, tile 16: horizontal tile pairs over all images
   int32_t pair;               // 1: the forward raster runs one warp per pair of tiles
   int32_t adjoint;            // the adjoint kernel of these views (gs_adjoint, resolved)
+  int32_t bwd_parts;          // tile and quadrant adjoints: parts of each tile's list
   int32_t n_gblocks;          // every image with m > 0: blocks of LR cells in all; else 0
   const float* grad_out0;     // direct: dL/dI of image 0
   float* grads0;              // direct: parameter gradients of image 0
