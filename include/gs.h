@@ -139,7 +139,8 @@ typedef enum { GS_BINNING_AUTO = 0, GS_BINNING_SORT = 1, GS_BINNING_GRID = 2 } g
 /* How the forward raster lays its warps over the screen tiles (a launch
  * parameter: the image is the same bit for bit):
  *   TILE: one warp per tile (tile 16: four strips of 4 columns, each walking
- *         the Gaussians whose window meets it);
+ *         the Gaussians whose window meets it; a team of 4 or 8 warps where the
+ *         lists are long and one warp would leave the chip idle);
  *   PAIR: one warp per horizontal pair of 16 x 16 tiles, in four strips of 8
  *         columns: the per-Gaussian work (shared-memory staging, operand
  *         loads) is shared by the two tiles. Needs GRID binning and tile 16

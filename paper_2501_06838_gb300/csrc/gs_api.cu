@@ -1,6 +1,7 @@
 // C-ABI entry points (include/gs.h): argument validation, workspace layout,
 // and the launch sequence of the render and its adjoint. All device work is
 // in the kernels of gs_preprocess.cu, gs_binning.cu and gs_raster.cu.
+#include <algorithm>
 #include <atomic>
 #include <cstdarg>
 #include <cmath>
@@ -250,6 +251,41 @@ int key_bits(int64_t tiles) {
 }
 int radix_passes(int64_t tiles) { return (key_bits(tiles) + 8) / 9; }
 
+// Warps per tile of the tile-16 forward: a team where lists are long (0: one
+// warp). A list's segments of 512 entries are what a team shares, so the rule
+// asks for lists of some segments: known from the views with the ratio window
+// (and the whole image, trunc_k <= 0); with k-sigma boxes only bounded below by
+// the Gaussians per tile, and then only where the tiles are few enough for all
+// teams to be resident at once (2 of 8 warps or 5 of 4 per SM, 152 SMs), where
+// idle warps take nobody's place. Measured, one warp -> team: 2,025 tiles with
+// lists of 23,000 3.73 -> 2.99 ms (8 warps: 3.11), 8,100 tiles with 6,400 3.08
+// -> 2.94 ms, 2,025 tiles with 1,500 320 -> 263 us, 250 tiles with 4,000 to
+// 10,000 547 -> 117 us (4 warps: 154), 256 tiles with 16 Gaussians per LR pixel
+// 115 -> 54 us; 625 tiles with lists of 80 14.2 -> 16.1 us, so those keep one.
+int team_of(const Problem& P, const gs_gaussians* g, const gs_view* v) {
+  if (P.tile != 16 || P.pair || P.batch == 64) return 0;
+  double listed = 0.0;
+  bool known = true;
+  for (int i = 0; i < P.n_images; ++i) {
+    const gs_view& V = v[i];
+    double nx = 1.0, ny = 1.0;   // tiles a window meets on average
+    if (!(V.trunc_k > 0.0f)) {
+      nx = (V.out_w + 15) / 16;
+      ny = (V.out_h + 15) / 16;
+    } else if (V.window == GS_WINDOW_RATIO) {
+      nx = std::min((V.out_w + 15) / 16.0, 1.0 + 2.0 * V.scale * V.trunc_k * V.lr_w / 16.0);
+      ny = std::min((V.out_h + 15) / 16.0, 1.0 + 2.0 * V.scale * V.trunc_k * V.lr_h / 16.0);
+    } else {
+      known = false;
+    }
+    listed += (double)g[i].n * nx * ny;
+  }
+  listed /= (double)P.tiles;
+  const bool few = P.tiles <= 760;
+  if (!(known ? listed >= (few ? 512.0 : 1024.0) : few && listed >= 128.0)) return 0;
+  return P.tiles <= 304 ? 8 : 4;
+}
+
 struct Call {
   Problem P;
   Layout L;
@@ -309,6 +345,7 @@ gs_status prepare(int32_t n_images, const gs_gaussians* g, const gs_view* v, voi
   }
   w.n_pairs = (int32_t)pairs;
   w.pair = c->P.pair;
+  w.team = team_of(c->P, g, v);
   w.adjoint = c->P.adjoint;
   // blocks of LR cells (the Gaussian-warp adjoint's block form), when
   // every image's Gaussians sit on a reference grid

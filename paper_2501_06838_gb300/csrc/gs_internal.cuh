@@ -111,6 +111,7 @@ struct Ws {
   int32_t direct;             // 1: one image, its grad_out / grads pointers below (adjoint)
   int32_t n_pairs;            // grid binning, tile 16: horizontal tile pairs over all images
   int32_t pair;               // 1: the forward raster runs one warp per pair of tiles
+  int32_t team;               // tile 16: warps of a team per tile in the forward raster (0: one warp)
   int32_t adjoint;            // the adjoint kernel of these views (gs_adjoint, resolved)
   int32_t bwd_parts;          // tile and quadrant adjoints: parts of each tile's list
   int32_t n_gblocks;          // every image with m > 0: blocks of LR cells in all; else 0

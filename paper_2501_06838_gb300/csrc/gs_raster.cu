@@ -84,6 +84,12 @@ __device__ __forceinline__ void load_ids(const uint32_t* vals, int bs, int nb, u
   }
 }
 
+// A tile's list is summed in segments of kSeg entries, one after the other:
+// out = ((S0 + S1) + S2) + .... One warp writes each segment's sums onto the
+// output as it ends; a team of warps sums them side by side and adds them in
+// the same order (k_raster_fwd_team): the same bits in every layout.
+constexpr int kSeg = 512;
+
 // Where a tile's Gaussian ids come from, one batch at a time (ids ascending,
 // so both sources give a tile the same Gaussians in the same order and the
 // forward the same bits).
@@ -123,15 +129,19 @@ struct Candidates {
   uint32_t gid, wrap;    // this lane's candidate; from a row's end to the next row's start
   int col;               // its position in its row
   uint32_t lo, hi;       // the region: (X0, Y0) and (X1, Y1)
-  __device__ __forceinline__ void start(int X0, int X1, int Y0, int Y1) {
-    const int lane = threadIdx.x & 31;
-    const int r = L > 0 ? lane / L : 0;
-    col = lane - r * L;
+  // to candidate `from` (lane 0's)
+  __device__ __forceinline__ void seek(int from) {
+    const int c = from + (int)(threadIdx.x & 31);
+    const int r = L > 0 ? c / L : 0;
+    col = c - r * L;
     gid = (uint32_t)(rb0 + (int64_t)r * rstride + col);
+    cur = from;
+  }
+  __device__ __forceinline__ void start(int X0, int X1, int Y0, int Y1) {
     wrap = (uint32_t)(rstride - L);
     lo = (uint32_t)(X0 & 0xffff) | ((uint32_t)Y0 << 16);
     hi = (uint32_t)(X1 & 0xffff) | ((uint32_t)Y1 << 16);
-    cur = 0;
+    seek(0);
   }
   // this lane's k-th candidate from cur on (none: a window that meets nothing)
   __device__ __forceinline__ uint2 load(int k) const {
@@ -181,7 +191,7 @@ struct GridSource {
       for (int k = 0; k < KR; ++k) {
         const bool hit = cand.meets(v[k]);
         const unsigned bal = __ballot_sync(0xffffffffu, hit);
-        if (threadIdx.x < 32 && hit)
+        if ((NT == 32 || threadIdx.x < 32) && hit)
           q[(tail + __popc(bal & ((1u << lane) - 1u))) & (QCAP - 1)] = g[k];
         tail += __popc(bal);
       }
@@ -191,7 +201,7 @@ struct GridSource {
     const int nb = min(BATCH, tail - head);
 #pragma unroll
     for (int j = 0; j < PF; ++j) {
-      const int i = j * NT + threadIdx.x;
+      const int i = j * NT + (NT == 32 ? lane : (int)threadIdx.x);
       gid[j] = i < nb ? q[(head + i) & (QCAP - 1)] : 0u;
     }
     head += nb;
@@ -464,7 +474,7 @@ __device__ __forceinline__ void walk_strips(StripAcc<NQ>& acc, StripMasks s, int
 template <int PF>
 __device__ __forceinline__ void issue_slots(const Ws& w, const uint32_t (&ids)[PF], int n,
                                             float4 (&raw)[PF][4 * 32]) {
-  const int lane = threadIdx.x;
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int j = 0; j < PF; ++j) {
     if (j * 32 + lane < n) {
@@ -507,6 +517,54 @@ __device__ __forceinline__ void store_strips(const ImageDesc* D, const StripAcc<
       }
     }
   }
+}
+
+// A segment's end (rare: its code is kept small): puts the region's pixels (16
+// NQ columns from ox, 16 rows from output row y0) through the table's shared
+// memory onto the output and clears them. go / add, the same over a tile's
+// lanes: whether the lane's tile is written, and whether onto what an earlier
+// segment left. (Every tile's last store taking this way as well cost 4% to 8%
+// of the forward.)
+template <int NQ>
+__device__ __forceinline__ void fold_strips(const ImageDesc* D, StripAcc<NQ>& acc,
+                                            StripTables<NQ>& t, int ox, int y0, bool go, bool add) {
+  constexpr int C = 16 * NQ, PLANE = 16 * C;
+  static_assert(sizeof(t.x) + sizeof(t.r) >= 3 * PLANE * sizeof(float), "the sums fit the table");
+  const int lane = threadIdx.x & 31, strip = lane >> 3, rp = lane & 7;
+  float* buf = reinterpret_cast<float*>(&t);
+  __syncwarp();
+  if (go) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int h = 0; h < NQ; ++h)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          float2& a = acc[j][2 * h][k];
+          float2& b = acc[j][2 * h + 1][k];
+          *reinterpret_cast<float4*>(buf + k * PLANE + (2 * rp + j) * C + 4 * (NQ * strip + h)) =
+              make_float4(a.x, a.y, b.x, b.y);
+          a = b = f2(0.0f, 0.0f);
+        }
+  }
+  __syncwarp();
+  const int H = D->out_h, W = D->out_w;
+  const int x = ox + lane % C;
+  if (go && x < W) {
+    float* o = D->out + (int64_t)y0 * W + x;
+#pragma unroll 1
+    for (int k = 0; k < 3; ++k, o += (int64_t)H * W) {
+#pragma unroll 4
+      for (int r = lane / C; r < 16; r += 32 / C) {
+        if (y0 + r >= H) break;
+        const float v = buf[k * PLANE + r * C + lane % C];
+        o[(int64_t)r * W] = add ? o[(int64_t)r * W] + v : v;
+      }
+    }
+  }
+  __syncwarp();
+  t.clear_front(lane);
+  __syncwarp();
 }
 
 template <int PF, bool GRID>
@@ -595,6 +653,8 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
   }
   for (int b = 0; b < nbat; ++b) {
     const int nb = min(BATCH, total - b * BATCH);
+    if (b > 0 && b % (kSeg / BATCH) == 0)
+      fold_strips<1>(D, acc, T[0], ox, oy - D->row0, true, b > kSeg / BATCH);   // a segment ends
     cp_async_wait_all();
     __syncwarp();
     StripMasks ms[PF];
@@ -611,7 +671,212 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
     __syncwarp();
   }
 
-  store_strips<1>(D, acc, ox + 4 * strip, oy - D->row0 + 2 * rp);
+  if (total > kSeg)
+    fold_strips<1>(D, acc, T[0], ox, oy - D->row0, true, true);
+  else
+    store_strips<1>(D, acc, ox + 4 * strip, oy - D->row0 + 2 * rp);
+}
+
+// ---------------------------------------------------------------------------
+// Forward of a 16 x 16 tile by a team of NW warps, for images of few tiles: the
+// warps sum the segments of the tile's list side by side, each as
+// k_raster_fwd16 does, and their sums are added in list order. In grid mode the
+// team first builds the tile's list together (each warp a run of the
+// candidates: count, prefix over the warps, write).
+//
+// What bounds it: the strips' arithmetic, once enough warps run. One warp per
+// tile left 2,025 tiles with lists of 23,000 at 3 or 4 warps per scheduler (the
+// fuller ones last: 3.73 ms; teams of four: 2.99) and 250 tiles with lists of
+// 4,000 to 10,000 waiting for the longest (514 us; teams of eight: 117). The
+// host's rule says where a team runs and what else was measured.
+// ---------------------------------------------------------------------------
+struct TeamWarp {
+  float4 raw[1][4 * 32];
+  StripTables<1> t;     // a segment's sums (768 floats) go to t.r once it is walked
+  uint32_t q[256];      // fallback enumeration (a list that did not fit)
+};
+static_assert(GridSource<32, 1>::QCAP == 256, "TeamWarp::q");
+static_assert(sizeof(StripTables<1>::r) >= 768 * sizeof(float), "segment sums");
+
+// The tile's list from the workspace (this launch may have written it).
+struct ListSource {
+  const uint32_t* list;
+  int pos, end;
+  __device__ __forceinline__ int next(uint32_t (&gid)[1]) {
+    const int nb = max(0, min(32, end - pos)), lane = threadIdx.x & 31;
+    gid[0] = lane < nb ? __ldcg(list + pos + lane) : 0u;
+    pos += nb;
+    return nb;
+  }
+};
+
+template <int NW, bool GRID>
+__global__ void __launch_bounds__(NW * 32) k_raster_fwd_team(Ws w, const uint32_t* vals) {
+  griddep_release();
+  griddep_wait();
+  constexpr int NT = NW * 32, PER = 768 / NT;
+  extern __shared__ float4 team_smem[];
+  TeamWarp* team = reinterpret_cast<TeamWarp*>(team_smem);
+  __shared__ int s_base, s_cnt[NW];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  TeamWarp& M = team[warp];
+  const ImageDesc* D;
+  int ox, oy;
+  tile_origin<16>(w, blockIdx.x, D, ox, oy);
+  const int strip = lane >> 3, rp = lane & 7;
+
+  int total;
+  const uint32_t* list;
+  bool listed = true;
+  GridSource<32, 1> cells;
+  if constexpr (GRID) {
+    grid_source_init<16, 32, 1>(w, D, ox, oy, M.q, cells);
+    // the tile's pair count: the prefix, along its tile row, of the footprint
+    // pass's per-row differences
+    const int lt = blockIdx.x - D->t_base;
+    const int tyl = lt / D->tiles_x, txl = lt - tyl * D->tiles_x;
+    const uint32_t* row = w.tcount + D->t_base + (int64_t)tyl * D->tiles_x;
+    uint32_t s = 0u;
+    for (int x = lane; x <= txl; x += 32) s += row[x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    total = (int)s;
+    if (threadIdx.x == 0) {
+      const unsigned long long b = atomicAdd(&w.hdr->list_cursor, (unsigned long long)total);
+      const bool fits = b + (unsigned long long)total <= (unsigned long long)w.capacity;
+      s_base = fits ? (int)b : -1;
+      w.ranges[blockIdx.x] = fits ? make_uint2((uint32_t)b, (uint32_t)(b + total)) : make_uint2(0u, 0u);
+      if (!fits && total > 0) atomicOr(&w.hdr->status, kStCapacity);
+    }
+    // this warp's run of candidates, counted
+    Candidates c = cells.cand;
+    const int run = ((c.total + NW * 128 - 1) / (NW * 128)) * 128;
+    const int c0 = min(c.total, warp * run);
+    c.total = min(c.total, c0 + run);
+    int cnt = 0;
+    for (c.seek(c0); c.cur < c.total; c.cur += 128) {
+      uint2 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) { v[k] = c.load(k); c.advance(); }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) cnt += __popc(__ballot_sync(0xffffffffu, c.meets(v[k])));
+    }
+    if (lane == 0) s_cnt[warp] = cnt;
+    __syncthreads();
+    int at = 0, all = 0;
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+      if (k == warp) at = all;
+      all += s_cnt[k];
+    }
+    if (all != total && threadIdx.x == 0) atomicOr(&w.hdr->status, kStInternal);
+    listed = s_base >= 0;
+    uint32_t* slice = w.vals[0] + (listed ? s_base : 0);
+    list = slice;
+    total = min(total, all);
+    if (listed) {
+      for (c.seek(c0); c.cur < c.total; c.cur += 128) {
+        uint2 v[4];
+        uint32_t g[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { g[k] = c.gid; v[k] = c.load(k); c.advance(); }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const bool hit = c.meets(v[k]);
+          const unsigned bal = __ballot_sync(0xffffffffu, hit);
+          const int i = at + __popc(bal & ((1u << lane) - 1u));
+          if (hit && i < total) slice[i] = g[k];
+          at += __popc(bal);
+        }
+      }
+      __syncthreads();   // the list is complete (and visible to the team)
+    }
+  } else {
+    const uint2 range = w.ranges[blockIdx.x];
+    list = vals + range.x;
+    total = (int)(range.y - range.x);
+  }
+
+  const int nseg = (total + kSeg - 1) / kSeg;
+  float sum[PER];   // of the values threadIdx.x + i * NT, value = channel * 256 + row * 16 + column
+#pragma unroll
+  for (int i = 0; i < PER; ++i) sum[i] = 0.0f;
+  int passed = 0;   // fallback: list entries enumerated so far
+  for (int first = 0; first < nseg; first += NW) {   // uniform over the team
+    const int seg = first + warp;
+    if (seg < nseg) {
+      StripAcc<1> acc;
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) acc[j][h][0] = acc[j][h][1] = acc[j][h][2] = f2(0.0f, 0.0f);
+      M.t.clear_front(lane);
+      const int lo = seg * kSeg, hi = min(total, lo + kSeg);
+      ListSource src{list, lo, hi};
+      uint32_t gid[1];
+      // the next batch: from the list, or (a list that did not fit) enumerated
+      // again, past the other warps' segments
+      auto next = [&]() -> int {
+        if (!GRID || listed) return src.next(gid);
+        if (passed >= hi) return 0;
+        int nb = cells.next(gid);
+        __syncwarp();
+        while (passed < lo && nb > 0) {
+          passed += nb;
+          nb = cells.next(gid);
+          __syncwarp();
+        }
+        passed += nb;
+        return nb;
+      };
+      int nb = next(), nn = 0;
+      if (nb > 0) {
+        issue_slots<1>(w, gid, nb, M.raw);
+        nn = next();
+      }
+      while (nb > 0) {
+        cp_async_wait_all();
+        __syncwarp();
+        const StripMasks ms =
+            strip_masks(stage_strips<1>(M.raw[0], lane, 31 - lane < nb, ox, oy, M.t), strip);
+        __syncwarp();
+        int n2 = 0;
+        if (nn > 0) {
+          issue_slots<1>(w, gid, nn, M.raw);
+          n2 = next();
+        }
+        walk_strips<1>(acc, ms, strip, rp, M.t);
+        __syncwarp();
+        nb = nn;
+        nn = n2;
+      }
+      float* ps = reinterpret_cast<float*>(M.t.r);
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          *reinterpret_cast<float4*>(ps + k * 256 + (2 * rp + j) * 16 + 4 * strip) =
+              make_float4(acc[j][0][k].x, acc[j][0][k].y, acc[j][1][k].x, acc[j][1][k].y);
+    }
+    __syncthreads();
+    const int n = min(NW, nseg - first);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      for (int k = 0; k < n; ++k) {
+        const float v = reinterpret_cast<const float*>(team[k].t.r)[threadIdx.x + i * NT];
+        sum[i] = first + k == 0 ? v : sum[i] + v;
+      }
+    }
+    __syncthreads();
+  }
+  const int H = D->out_h, W = D->out_w;
+  const int64_t plane = (int64_t)H * W;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const int v = threadIdx.x + i * NT;
+    const int x = ox + (v & 15), y = oy - D->row0 + ((v >> 4) & 15);
+    if (x < W && y < H) D->out[(v >> 8) * plane + (int64_t)y * W + x] = sum[i];
+  }
 }
 
 template <int TILE, int BY, int PF, bool GRID>
@@ -773,8 +1038,10 @@ struct PairSource {
   uint8_t* qf;           // shared [QCAP] hit flags: 1 tile A, 2 tile B
   Candidates cand;       // of the pair's region
   int head, tail, XM;    // tile A [X0, XM - 1], tile B [XM, X1]
-  // the next batch: ids and flags of up to BATCH kept candidates, gid order
-  __device__ __forceinline__ int next(uint32_t (&gid)[PF], uint32_t (&fl)[PF]) {
+  // the next batch: ids and flags of up to BATCH kept candidates, gid order, at
+  // most room_a of them in tile A and room_b in tile B
+  __device__ __forceinline__ int next(uint32_t (&gid)[PF], uint32_t (&fl)[PF], int room_a,
+                                      int room_b) {
     const int lane = threadIdx.x & 31;
     while (tail - head < BATCH && cand.cur < cand.total) {
       uint32_t g[KR];
@@ -800,13 +1067,25 @@ struct PairSource {
       cand.cur += 32 * KR;
     }
     __syncwarp();
-    const int nb = min(BATCH, tail - head);
+    int nb = min(BATCH, tail - head);
+    const int n = nb;
 #pragma unroll
     for (int j = 0; j < PF; ++j) {
       const int i = j * NT + lane;
       const int at = (head + i) & (QCAP - 1);
-      gid[j] = i < nb ? q[at] : 0u;
-      fl[j] = i < nb ? (uint32_t)qf[at] : 0u;
+      gid[j] = i < n ? q[at] : 0u;
+      fl[j] = i < n ? (uint32_t)qf[at] : 0u;
+      if (min(room_a, room_b) < 32) {   // a segment may end inside: the batch ends with it
+        const unsigned ba = __ballot_sync(0xffffffffu, fl[j] & 1u);
+        const unsigned bb = __ballot_sync(0xffffffffu, fl[j] & 2u);
+        if (__popc(ba) > room_a) nb = min(nb, j * NT + (int)__fns(ba, 0, room_a + 1));
+        if (__popc(bb) > room_b) nb = min(nb, j * NT + (int)__fns(bb, 0, room_b + 1));
+        room_a = max(0, room_a - __popc(ba));
+        room_b = max(0, room_b - __popc(bb));
+      } else {
+        room_a -= 32;
+        room_b -= 32;
+      }
     }
     head += nb;
     __syncwarp();
@@ -911,16 +1190,34 @@ __global__ void __launch_bounds__(32, 16) k_raster_fwd_pair(Ws w) {
 #pragma unroll
   for (int j = 0; j < PF; ++j) T[j].clear_front(lane);
 
+  auto next = [&](uint32_t (&ids)[PF], uint32_t (&fl)[PF]) {
+    return src.next(ids, fl, kSeg - (pos_a & (kSeg - 1)), kSeg - (pos_b & (kSeg - 1)));
+  };
   uint32_t gid[PF], fl[PF];
-  int nb0 = src.next(gid, fl);   // batch 0
+  int nb0 = next(gid, fl);   // batch 0
   keep(gid, fl, nb0);
+  int next_a = pos_a, next_b = pos_b;   // the two lists' entries up to and with batch b
   int nb1 = 0;
   if (nb0 > 0) {
     issue_slots<PF>(w, gid, nb0, raw);
-    nb1 = src.next(gid, fl);      // batch 1
+    nb1 = next(gid, fl);      // batch 1
     keep(gid, fl, nb1);
   }
+  int done_a = 0, done_b = 0;         // list entries of the two tiles summed so far
+  int written_a = 0, written_b = 0;   // ... and already on the output
   while (nb0 > 0) {
+    const bool end_a = done_a > written_a && (done_a & (kSeg - 1)) == 0;   // a segment ends
+    const bool end_b = done_b > written_b && (done_b & (kSeg - 1)) == 0;
+    if (end_a || end_b) {
+      fold_strips<2>(D, acc, T[0], ox, oy - D->row0, strip < 2 ? end_a : end_b,
+                     (strip < 2 ? written_a : written_b) > 0);
+      if (end_a) written_a = done_a;
+      if (end_b) written_b = done_b;
+    }
+    done_a = next_a;
+    done_b = next_b;
+    next_a = pos_a;
+    next_b = pos_b;
     cp_async_wait_all();
     __syncwarp();
     StripMasks ms[PF];
@@ -931,7 +1228,7 @@ __global__ void __launch_bounds__(32, 16) k_raster_fwd_pair(Ws w) {
     int nb2 = 0;
     if (nb1 > 0) {
       issue_slots<PF>(w, gid, nb1, raw);
-      nb2 = src.next(gid, fl);    // batch b + 2
+      nb2 = next(gid, fl);    // batch b + 2
       keep(gid, fl, nb2);
     }
 #pragma unroll
@@ -944,7 +1241,10 @@ __global__ void __launch_bounds__(32, 16) k_raster_fwd_pair(Ws w) {
     if (lane == 0) atomicOr(&w.hdr->status, kStInternal);
   }
 
-  store_strips<2>(D, acc, ox + 8 * strip, oy - D->row0 + 2 * rp);
+  if (written_a + written_b > 0)
+    fold_strips<2>(D, acc, T[0], ox, oy - D->row0, true, (strip < 2 ? written_a : written_b) > 0);
+  else
+    store_strips<2>(D, acc, ox + 8 * strip, oy - D->row0 + 2 * rp);
 }
 
 template <int TILE, int BY, int PF>
@@ -960,6 +1260,18 @@ cudaError_t run16(const Ws& w, const uint32_t* vals, cudaStream_t s) {
   LaunchScope ls(kKRasterFwd, s);
   if (w.grid) return launch_chain(k_raster_fwd16<PF, true>, dim3(w.tiles), dim3(32), 0, s, w, vals);
   return launch_chain(k_raster_fwd16<PF, false>, dim3(w.tiles), dim3(32), 0, s, w, vals);
+}
+
+template <int NW>
+cudaError_t run_team(const Ws& w, const uint32_t* vals, cudaStream_t s) {
+  constexpr size_t smem = NW * sizeof(TeamWarp);
+  auto kernel = w.grid ? k_raster_fwd_team<NW, true> : k_raster_fwd_team<NW, false>;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  LaunchScope ls(kKRasterFwd, s);
+  return launch_chain(kernel, dim3(w.tiles), dim3(NW * 32), smem, s, w, vals);
 }
 
 // Launch configurations: tile edge -> rows per thread (threads = TILE^2 / BY);
@@ -979,6 +1291,7 @@ cudaError_t dispatch(const Ws& w, const uint32_t* vals, int batch, cudaStream_t 
     case 32:  // 64 threads
       return batch >= 128 ? run<32, 16, 2>(w, vals, s) : run<32, 16, 1>(w, vals, s);
     default:  // 32 threads
+      if (w.team) return w.team > 4 ? run_team<8>(w, vals, s) : run_team<4>(w, vals, s);
       return batch >= 64 ? run16<2>(w, vals, s) : run16<1>(w, vals, s);
   }
 }
