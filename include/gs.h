@@ -102,11 +102,10 @@ typedef enum { GS_ALIGN_EQ4 = 0, GS_ALIGN_HALF = 1 } gs_align;
  *             ref_grid_m > 0 the warps work in CTAs over 8 x 8 blocks of LR
  *             cells, with the upstream gradient under the block staged in
  *             shared memory; the sums are the same);
- *   QUADRANT: TILE over the 8 x 8 quadrants of 16 x 16 tiles: each quadrant's
- *             warp keeps, from the tile's list, the Gaussians whose window
- *             meets the quadrant, so small windows waste fewer pixel
- *             evaluations at tile edges. Needs tile 16 (GS_ERR_UNSUPPORTED
- *             otherwise);
+ *   QUADRANT: TILE over the 8 x 8 quadrants of 16 x 16 tiles: a CTA per tile
+ *             walks the (Gaussian, quadrant) pairs whose window meets the
+ *             quadrant, so small windows waste fewer pixel evaluations at tile
+ *             edges. Needs tile 16 (GS_ERR_UNSUPPORTED otherwise);
  *   AUTO:     QUADRANT at tile 16 when every view uses the SIGMA window with
  *             trunc_k > 0 at scale < 6 (small windows, where it measured
  *             faster), else TILE

@@ -206,55 +206,201 @@ __device__ __forceinline__ void bwd_one_tile(const Ws& w, const uint32_t* vals, 
   }
 }
 
-// The adjoint of quadrant q (0..3, row-major) of 16 x 16 tile t by one warp:
-// the tile's list is filtered to the Gaussians whose window meets the 8 x 8
-// quadrant (a ballot per 32 entries into a shared queue of at most 63 ids),
-// and the quadrant is evaluated in chunks of 32 of those. Every pixel pair the
-// tile-16 walk would evaluate for a Gaussian that misses the quadrant is
-// skipped, at the cost of reading the tile's list and windows four times.
+// The adjoint over blocks of 8 columns x kBh rows of 16 x 16 tiles, for small
+// windows: a CTA of kBwWarps warps takes a tile (or one part of its list). It
+// stages the tile's upstream gradient and, 32 kBwWarps list entries at a time,
+// the entries' records in shared memory, lists the (entry, block) items whose
+// window meets the block (block by block, entries in list order) and walks the
+// items in chunks of 32, one per lane: each lane evaluates its own Gaussian
+// over its own block, so chunks are full across blocks, and a chunk waits on
+// shared memory only. Lanes of a chunk are in at most 16 / kBh * 2 blocks, so
+// a step's gradient loads touch that many addresses; rows of blocks are padded
+// apart to keep those in different banks. Each item ends in two 16-byte
+// reductions to its Gaussian's accumulator.
+//
+// What bounds it: the FP32 pipe (58% busy in the profile; FFMA2s with three
+// operands take 2.3 to 2.9 cycles, so 70% to 80% of what it can do), then the
+// pixels of blocks outside the windows. Against one warp per quadrant, which
+// filtered the tile's list and fetched each chunk's records from L2 by itself
+// and ran its last chunk 40% empty: 53.8 -> 43.8 us on 65,536 Gaussians at
+// 1024 x 1024, 86 -> 76 us on 220,052 at 1002 x 751, 55.7 -> 48.0 us on 100,000
+// at absolute centres. Blocks of 4 rows evaluate fewer pixels but fold twice as
+// often: 44.8, 73.7 and 48.6 us. Two warps per CTA: 49.3, 84.4 and 55.9 us;
+// eight: 59.9, 81.0 and 52.2 us.
+constexpr int kBh = 8;
+constexpr int kBwWarps = 4;
+constexpr int kBlocksX = 2, kBlocksY = 16 / kBh, kBlocks = kBlocksX * kBlocksY;
+constexpr int kBwPad = kBh == 8 ? 2 : 1;   // entries between two rows of blocks
+
+struct BlockSmem {
+  float4 gA[128 + kBwPad * kBlocksY];   // gradient, as stage_grad's sgA / sgB, padded
+  float2 gB[128 + kBwPad * kBlocksY];
+  float4 rec[kRecordF4][32 * kBwWarps];
+  uint16_t item[kBlocks * 32 * kBwWarps];   // entry | block << 8
+  int cnt[kBwWarps][kBlocks];
+  uint32_t gid[32 * kBwWarps];
+};
+
+// One chunk of items: the lane's Gaussian (entry e of the staged records) over
+// the lane's block q, as bwd_chunk does over a whole tile.
+__device__ __forceinline__ void bwd_block(const Ws& w, const BlockSmem& S, int e, int q, bool valid,
+                                          int tox, int toy) {
+  const int bx = 8 * (q % kBlocksX), by = kBh * (q / kBlocksX);
+  const int ox = tox + bx, oy = toy + by;
+  float cxl = 0.f, cyl = 0.f, sA = 0.f, sK = 0.f, gy2 = 0.f, l = 0.f, cr = 0.f, cg = 0.f, cb = 0.f;
+  int lx0 = 1, lx1 = 0, ly0 = kBh, ly1 = -1;
+  if (valid) {
+    const float4 f0 = S.rec[0][e], f1 = S.rec[1][e], f2 = S.rec[2][e], f3 = S.rec[3][e];
+    cxl = __fadd_rn(__fsub_rn(f0.x, (float)ox), f0.y);
+    cyl = __fadd_rn(__fsub_rn(f0.z, (float)oy), f0.w);
+    sA = f1.x; sK = f1.y; gy2 = f1.z; l = f1.w;
+    cr = f2.x; cg = f2.y; cb = f2.z;
+    lx0 = __float_as_int(f3.x) - ox;
+    lx1 = __float_as_int(f3.y) - ox;
+    ly0 = max(__float_as_int(f3.z) - oy, 0);
+    ly1 = min(__float_as_int(f3.w) - oy, kBh - 1);
+  }
+  // rows some lane's window reaches
+  const int rlo = __reduce_min_sync(0xffffffffu, ly0);
+  const int rhi = __reduce_max_sync(0xffffffffu, ly1);
+  const float2 cr2 = p2(cr, cr), cg2 = p2(cg, cg), cb2 = p2(cb, cb), nsK2 = p2(-sK, -sK);
+  float2 Cr = p2(0.f, 0.f), Cg = Cr, Cb = Cr;
+  float Sd = 0.f, SY = 0.f, Sdd = 0.f, SdY = 0.f, SYY = 0.f;
+  float2 Xs2[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c0 = 2 * j, c1 = c0 + 1;
+    const float a = __fsub_rn((float)c0, cxl), b = __fsub_rn((float)c1, cxl);
+    Xs2[j] = p2((c0 >= lx0 && c0 <= lx1) ? sA * a : kFarG, (c1 >= lx0 && c1 <= lx1) ? sA * b : kFarG);
+  }
+  const int at = by * 8 + bx / 2 + kBwPad * (q / kBlocksX);
+  const float4* ga = S.gA + at;
+  const float2* gb = S.gB + at;
+  for (int r = rlo; r <= rhi; ++r) {
+    const float Y = __fsub_rn((float)r, cyl);
+    const float R = (r >= ly0 && r <= ly1) ? fmaf(gy2 * Y, Y, l) : -kInfG;
+    const float2 Y2 = p2(Y, Y), R2 = p2(R, R);
+    float2 A0, A1, A2;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float4 v = ga[r * 8 + j];
+      const float2 gbj = gb[r * 8 + j];
+      const float2 gr2 = p2(v.x, v.y), gg2 = p2(v.z, v.w);
+      const float2 d = __ffma2_rn(nsK2, Y2, Xs2[j]);   // one rounding: d cancels for |rho| -> 1
+      const float2 ex = __ffma2_rn(p2(-d.x, -d.y), d, R2);
+      const float2 wv = p2(ex2_approx(ex.x), ex2_approx(ex.y));
+      const float2 G = __ffma2_rn(gbj, cb2, __ffma2_rn(gg2, cg2, __fmul2_rn(gr2, cr2)));
+      Cr = __ffma2_rn(gr2, wv, Cr);
+      Cg = __ffma2_rn(gg2, wv, Cg);
+      Cb = __ffma2_rn(gbj, wv, Cb);
+      const float2 Gw = __fmul2_rn(G, wv);
+      const float2 Gwd = __fmul2_rn(Gw, d);
+      if (j == 0) {
+        A0 = Gw;
+        A1 = Gwd;
+        A2 = __fmul2_rn(Gwd, d);
+      } else {
+        A0 = __fadd2_rn(A0, Gw);
+        A1 = __fadd2_rn(A1, Gwd);
+        A2 = __ffma2_rn(Gwd, d, A2);
+      }
+    }
+    const float a0 = A0.x + A0.y, a1 = A1.x + A1.y, a2 = A2.x + A2.y;
+    const float ty = Y * a0;
+    SY += ty;
+    SYY = fmaf(ty, Y, SYY);
+    Sd += a1;
+    SdY = fmaf(Y, a1, SdY);
+    Sdd += a2;
+  }
+  if (valid) {   // two 16-byte reductions; rows of 12 floats are 16-byte aligned
+    float4* acc = reinterpret_cast<float4*>(w.grec + (int64_t)S.gid[e] * 12);
+    atomicAdd(acc, make_float4(Sd, SY, Sdd, SdY));
+    atomicAdd(acc + 1, make_float4(SYY, Cr.x + Cr.y, Cg.x + Cg.y, Cb.x + Cb.y));
+  }
+}
+
 template <bool SPLIT>
-__device__ __forceinline__ void bwd_one_quadrant(const Ws& w, const uint32_t* vals, int t, int part,
-                                                 int q, float4* sgA, float2* sgB, uint32_t* qids) {
+__global__ void __launch_bounds__(32 * kBwWarps) k_raster_bwd_quad(Ws w, const uint32_t* vals) {
+  griddep_release();
+  griddep_wait();
+  constexpr int NT = 32 * kBwWarps;
+  __shared__ BlockSmem S;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t = SPLIT ? (int)(blockIdx.x / (uint32_t)w.bwd_parts) : (int)blockIdx.x;
   const uint2 range = w.ranges[t];
-  int lo, n;
-  if (!list_part<SPLIT>(w, range, part, lo, n)) return;   // no entry (uniform)
-  const int lane = threadIdx.x;
+  int lo, hi;
+  if (!list_part<SPLIT>(w, range, SPLIT ? (int)blockIdx.x - t * w.bwd_parts : 0, lo, hi)) return;
   const int im = image_of_tile(w.images, w.n_images, t);
   const ImageDesc* D = &w.images[im];
   const int lt = t - D->t_base;
   const int tyi = lt / D->tiles_x;
-  const int ox = (lt - tyi * D->tiles_x) * 16 + (q & 1) * 8;
-  const int oy = tyi * 16 + D->row0 + (q >> 1) * 8;
-  if (ox >= D->out_w || oy - D->row0 >= D->out_h) return;   // quadrant past the output (uniform)
-  stage_grad<8>(w, D, ox, oy, sgA, sgB);
-  const int4* win = reinterpret_cast<const int4*>(w.records);   // f3 of each record
-  int head = 0, pos = lo;
-  // list entries pos .. pos + 31, loaded one top-up ahead of their window test
-  uint32_t nid = pos + lane < n ? __ldg(vals + range.x + pos + lane) : 0xffffffffu;
-  while (true) {
-    // top up the queue to at least 32 ids (or the end of the list)
-    while (head < 32 && pos < n) {
-      const uint32_t gid = nid;
-      pos += 32;
-      nid = pos + lane < n ? __ldg(vals + range.x + pos + lane) : 0xffffffffu;
-      bool meets = false;
-      if (gid < (uint32_t)w.n) {
-        const int4 b = __ldg(win + (int64_t)gid * kRecordF4 + 3);   // x0, x1, y0, y1 (image)
-        meets = b.x <= ox + 7 && b.y >= ox && b.z <= oy + 7 && b.w >= oy;
-      }
-      const uint32_t m = __ballot_sync(0xffffffffu, meets);
-      if (meets) qids[head + __popc(m & ((1u << lane) - 1u))] = gid;
-      head += __popc(m);
+  const int ox = (lt - tyi * D->tiles_x) * 16;
+  const int oy = tyi * 16 + D->row0;
+  {
+    const int H = D->out_h, W = D->out_w;
+    const int64_t plane = (int64_t)H * W;
+    const float* go = w.direct ? w.grad_out0 : D->grad_out;
+    float* fa = reinterpret_cast<float*>(S.gA);
+    float* fb = reinterpret_cast<float*>(S.gB);
+#pragma unroll
+    for (int idx = threadIdx.x; idx < 256; idx += NT) {
+      const int r = idx >> 4, x = idx & 15;
+      const int gx = ox + x, gy = oy - D->row0 + r;
+      const bool in = gx < W && gy < H;
+      const int64_t o = in ? (int64_t)gy * W + gx : 0;   // always a valid address
+      const float vr = __ldg(go + o), vg = __ldg(go + plane + o), vb = __ldg(go + 2 * plane + o);
+      const int e = r * 8 + (x >> 1) + kBwPad * (r / kBh), hb = x & 1;
+      fa[4 * e + hb] = in ? vr : 0.0f;
+      fa[4 * e + 2 + hb] = in ? vg : 0.0f;
+      fb[2 * e + hb] = in ? vb : 0.0f;
     }
-    __syncwarp();
-    if (head == 0) break;   // uniform: the list is exhausted
-    const uint32_t gid = lane < head ? qids[lane] : 0xffffffffu;
-    const uint32_t carry = lane + 32 < head ? qids[lane + 32] : 0u;
-    __syncwarp();
-    if (lane + 32 < head) qids[lane] = carry;   // the ids past this chunk move to the front
-    head = head > 32 ? head - 32 : 0;
-    __syncwarp();
-    bwd_chunk<8>(w, gid, gid < (uint32_t)w.n, ox, oy, sgA, sgB);
+  }
+  for (int base = lo; base < hi; base += NT) {
+    // this thread's entry: its record, and the blocks its window meets
+    const int i = base + (int)threadIdx.x;
+    const uint32_t gid = i < hi ? __ldg(vals + range.x + i) : 0xffffffffu;
+    uint32_t meets = 0u;
+    if (gid < (uint32_t)w.n) {   // the list holds Gaussian ids
+      const float4* rec = w.records + (int64_t)gid * kRecordF4;
+      const float4 f0 = rec[0], f1 = rec[1], f2 = rec[2], f3 = rec[3];
+      S.rec[0][threadIdx.x] = f0;
+      S.rec[1][threadIdx.x] = f1;
+      S.rec[2][threadIdx.x] = f2;
+      S.rec[3][threadIdx.x] = f3;
+      S.gid[threadIdx.x] = gid;
+      const int x0 = __float_as_int(f3.x) - ox, x1 = __float_as_int(f3.y) - ox;
+      const int y0 = __float_as_int(f3.z) - oy, y1 = __float_as_int(f3.w) - oy;
+#pragma unroll
+      for (int q = 0; q < kBlocks; ++q) {
+        const int bx = 8 * (q % kBlocksX), by = kBh * (q / kBlocksX);
+        if (x0 <= bx + 7 && x1 >= bx && y0 <= by + kBh - 1 && y1 >= by) meets |= 1u << q;
+      }
+    }
+    uint32_t bal[kBlocks];
+#pragma unroll
+    for (int q = 0; q < kBlocks; ++q) {
+      bal[q] = __ballot_sync(0xffffffffu, (meets >> q) & 1u);
+      if (lane == 0) S.cnt[warp][q] = __popc(bal[q]);
+    }
+    __syncthreads();
+    int items = 0;
+#pragma unroll
+    for (int q = 0; q < kBlocks; ++q) {
+#pragma unroll
+      for (int k = 0; k < kBwWarps; ++k) {
+        if (k == warp && ((meets >> q) & 1u))
+          S.item[items + __popc(bal[q] & ((1u << lane) - 1u))] = (uint16_t)(threadIdx.x | (q << 8));
+        items += S.cnt[k][q];
+      }
+    }
+    __syncthreads();
+    for (int c = 32 * warp; c < items; c += NT) {
+      const bool valid = c + lane < items;
+      const int it = valid ? S.item[c + lane] : 0;
+      bwd_block(w, S, it & 0xff, it >> 8, valid, ox, oy);
+    }
+    if (base + NT < hi) __syncthreads();   // every warp is done with the records and the items
   }
 }
 
@@ -285,51 +431,42 @@ __global__ void __launch_bounds__(32, 32) k_raster_bwd_tile(Ws w, const uint32_t
   }
 }
 
-// The same over the 8 x 8 quadrants of 16 x 16 tiles: unit u is quadrant
-// u % 4 of tile u / 4, so the four quadrants of a tile run side by side.
-template <bool SPLIT>
-__global__ void __launch_bounds__(32) k_raster_bwd_quad(Ws w, const uint32_t* vals) {
-  griddep_release();
-  griddep_wait();
-  __shared__ float4 sgA[32];
-  __shared__ float2 sgB[32];
-  __shared__ uint32_t qids[64];
-  const uint32_t parts = SPLIT ? (uint32_t)w.bwd_parts : 1u, units = 4u * (uint32_t)w.tiles * parts;
-  const bool more = gridDim.x < units;   // uniform over the grid
-  uint32_t cur = blockIdx.x;
-  while (cur < units) {
-    const uint32_t v = cur >> 2, t = v / parts;
-    bwd_one_quadrant<SPLIT>(w, vals, (int)t, (int)(v - t * parts), (int)(cur & 3u), sgA, sgB, qids);
-    if (!more) break;
-    uint32_t nx = 0;
-    if (threadIdx.x == 0) nx = gridDim.x + atomicAdd(&w.hdr->bwd_counter, 1u);
-    cur = __shfl_sync(0xffffffffu, nx, 0);
-    __syncwarp();   // every lane is done with the staged gradient and the queue
-  }
-}
-
 }  // namespace
 
 namespace {
 
-// One launch of a tile or quadrant adjoint over `units` tiles (or quadrants).
-// Where they fill at most half of the CTAs that are resident at once, one warp
-// per unit leaves the chip idle while the longest lists are walked: every list
-// is then cut into parts (whole chunks of 32 entries, at most kBwdParts) that
-// fill the chip twice over. Measured, 4 images of 48 x 48 LR pixels with 16
-// Gaussians each (250 tiles, lists of 4,000 to 10,000): 656 -> 86 us (parts
-// that fill the chip once: 106). A part stages the unit's gradient again and
-// cuts a quadrant's queue short, so a fuller chip keeps whole lists: 16 crops
-// with 3,600 quadrants, short lists, took 38.7 us in parts against 37.1.
-cudaError_t launch_bwd(void (*whole)(Ws, const uint32_t*), void (*split)(Ws, const uint32_t*), Ws w,
-                       int64_t units, const uint32_t* lists, cudaStream_t s) {
+// Parts each tile's list is cut into. Where the tiles fill at most half of the
+// CTAs that are resident at once (`full`), one CTA per tile leaves the chip idle
+// while the longest lists are walked: every list is then cut into parts (whole
+// chunks of 32 entries, at most kBwdParts) that fill the chip twice over.
+// Measured, 4 images of 48 x 48 LR pixels with 16 Gaussians each (250 tiles,
+// lists of 4,000 to 10,000): 656 -> 86 us (parts that fill the chip once: 106).
+// A part stages the tile's gradient again and leaves a chunk short, so a fuller
+// chip keeps whole lists: 16 crops with short lists took 38.7 us in parts
+// against 37.1.
+int32_t list_parts(int64_t tiles, int64_t full) {
+  return 2 * tiles > full ? 1 : (int32_t)std::min<int64_t>(kBwdParts, (2 * full + tiles - 1) / tiles);
+}
+
+// The tile adjoint: a persistent launch of one-warp CTAs.
+cudaError_t launch_tile(void (*whole)(Ws, const uint32_t*), void (*split)(Ws, const uint32_t*), Ws w,
+                        const uint32_t* lists, cudaStream_t s) {
   const int64_t full = resident_grid((const void*)whole, 32, INT32_MAX);
-  w.bwd_parts = 1;
-  if (2 * units > full)
-    return launch_chain(whole, dim3((unsigned)std::min(full, units)), dim3(32), 0, s, w, lists);
-  w.bwd_parts = (int32_t)std::min<int64_t>(kBwdParts, (2 * full + units - 1) / units);
-  const int64_t ctas = resident_grid((const void*)split, 32, units * w.bwd_parts);
+  w.bwd_parts = list_parts(w.tiles, full);
+  if (w.bwd_parts == 1)
+    return launch_chain(whole, dim3((unsigned)std::min<int64_t>(full, w.tiles)), dim3(32), 0, s, w, lists);
+  const int64_t ctas = resident_grid((const void*)split, 32, (int64_t)w.tiles * w.bwd_parts);
   return launch_chain(split, dim3((unsigned)ctas), dim3(32), 0, s, w, lists);
+}
+
+// The quadrant adjoint: a CTA per tile, or per part of a tile's list.
+cudaError_t launch_quad(Ws w, const uint32_t* lists, cudaStream_t s) {
+  const dim3 block(32 * kBwWarps);
+  w.bwd_parts = list_parts(w.tiles, resident_grid((const void*)k_raster_bwd_quad<false>,
+                                                  32 * kBwWarps, INT32_MAX));
+  const dim3 grid((unsigned)((int64_t)w.tiles * w.bwd_parts));
+  if (w.bwd_parts == 1) return launch_chain(k_raster_bwd_quad<false>, grid, block, 0, s, w, lists);
+  return launch_chain(k_raster_bwd_quad<true>, grid, block, 0, s, w, lists);
 }
 
 }  // namespace
@@ -338,18 +475,11 @@ cudaError_t launch_raster_bwd_tile(const Ws& w, const uint32_t* lists, bool quad
                                    cudaStream_t s) {
   if (w.tiles == 0) return cudaSuccess;
   LaunchScope ls(kKRasterBwd, s);
-  if (quadrants)   // tile 16 (the caller checks)
-    return launch_bwd(k_raster_bwd_quad<false>, k_raster_bwd_quad<true>, w, 4 * (int64_t)w.tiles,
-                      lists, s);
+  if (quadrants) return launch_quad(w, lists, s);   // tile 16 (the caller checks)
   switch (w.tile) {
-    case 8:
-      return launch_bwd(k_raster_bwd_tile<8, false>, k_raster_bwd_tile<8, true>, w, w.tiles, lists, s);
-    case 32:
-      return launch_bwd(k_raster_bwd_tile<32, false>, k_raster_bwd_tile<32, true>, w, w.tiles, lists,
-                        s);
-    default:
-      return launch_bwd(k_raster_bwd_tile<16, false>, k_raster_bwd_tile<16, true>, w, w.tiles, lists,
-                        s);
+    case 8: return launch_tile(k_raster_bwd_tile<8, false>, k_raster_bwd_tile<8, true>, w, lists, s);
+    case 32: return launch_tile(k_raster_bwd_tile<32, false>, k_raster_bwd_tile<32, true>, w, lists, s);
+    default: return launch_tile(k_raster_bwd_tile<16, false>, k_raster_bwd_tile<16, true>, w, lists, s);
   }
 }
 
