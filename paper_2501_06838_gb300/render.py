@@ -104,10 +104,9 @@ def _device(gs: Sequence[Gaussians], stream=None) -> torch.device:
     dev = gs[0].rho.device
     if dev.type != "cuda":
         raise ValueError("parameter tensors must be CUDA tensors")
-    for g in gs:
-        for t in g.tensors():
-            if t.device != dev:
-                raise ValueError(f"all parameter tensors must be on one device ({dev}, {t.device})")
+    for g in gs:   # (one image's tensors share a device: _struct_g)
+        if g.rho.device != dev:
+            raise ValueError(f"all parameter tensors must be on one device ({dev}, {g.rho.device})")
     sdev = stream.device if stream is not None else torch.device("cuda", torch.cuda.current_device())
     if sdev != dev:
         raise ValueError(f"parameters are on {dev} but the launch stream is on {sdev}; "
@@ -115,13 +114,9 @@ def _device(gs: Sequence[Gaussians], stream=None) -> torch.device:
     return dev
 
 
-def _struct_g(g: Gaussians) -> _abi.GsGaussians:
-    ts = g.tensors()
+def _refuse(ts, shapes):
+    """The error for parameter tensors that are not what a call takes."""
     dt = ts[0].dtype
-    if dt not in _DTYPES:
-        raise TypeError(f"unsupported parameter dtype {dt}")
-    n = g.n
-    shapes = ((n, 2), (n, 2), (n,), (n, 3), (n,))
     for t, shp in zip(ts, shapes):
         if t.dtype != dt:
             raise TypeError("all parameter tensors must share one dtype")
@@ -131,36 +126,67 @@ def _struct_g(g: Gaussians) -> _abi.GsGaussians:
             raise ValueError("all parameter tensors must be on one device")
         if not t.is_contiguous() or tuple(t.shape) != shp:
             raise ValueError(f"parameter tensor must be contiguous with shape {shp}, got {tuple(t.shape)}")
-    hp = None
-    if g.head is not None:
-        h = g.head
-        hp = ctypes.pointer(_abi.GsHead(float(h.sigma_lo), float(h.sigma_span), float(h.rho_scale),
-                                        float(h.offset_scale), int(h.offset_tanh)))
-    G = _abi.GsGaussians(ts[0].data_ptr(), ts[1].data_ptr(), ts[2].data_ptr(),
-                         ts[3].data_ptr(), ts[4].data_ptr(), n, _DTYPES[dt], int(g.ref_grid_m), hp)
+
+
+def _head_struct(h):
+    return ctypes.pointer(_abi.GsHead(float(h.sigma_lo), float(h.sigma_span), float(h.rho_scale),
+                                      float(h.offset_scale), int(h.offset_tanh)))
+
+
+def _fields_g(g: Gaussians, hp) -> tuple:
+    """The checked fields of one image's gs_gaussians (hp: its head's struct or None)."""
+    o, s, r, c, a = ts = g.tensors()
+    dt, dev = o.dtype, o.device
+    code = _DTYPES.get(dt)
+    if code is None:
+        raise TypeError(f"unsupported parameter dtype {dt}")
+    n = int(r.shape[0])
+    shapes = ((n, 2), (n, 2), (n,), (n, 3), (n,))
+    if not (o.is_cuda and s.dtype == dt and r.dtype == dt and c.dtype == dt and a.dtype == dt
+            and s.device == dev and r.device == dev and c.device == dev and a.device == dev
+            and (o.shape, s.shape, r.shape, c.shape, a.shape) == shapes
+            and o.is_contiguous() and s.is_contiguous() and r.is_contiguous()
+            and c.is_contiguous() and a.is_contiguous()):
+        _refuse(ts, shapes)
+    return (o.data_ptr(), s.data_ptr(), r.data_ptr(), c.data_ptr(), a.data_ptr(), n, code,
+            int(g.ref_grid_m), hp)
+
+
+def _struct_g(g: Gaussians) -> _abi.GsGaussians:
+    hp = None if g.head is None else _head_struct(g.head)
+    G = _abi.GsGaussians(*_fields_g(g, hp))
     G._head_keep = hp   # the C struct points into this object during the call
     return G
 
 
+def _fields_v(v, tile: int = 0, batch: int = 0, adjoint: int = 0) -> tuple:
+    return (int(v.lr_h), int(v.lr_w), int(v.out_h), int(v.out_w), float(v.scale),
+            float(getattr(v, "trunc_k", 3.0)), int(getattr(v, "norm", 0)),
+            int(tile or getattr(v, "tile", 0) or 0), int(batch or getattr(v, "batch", 0) or 0),
+            int(getattr(v, "window", 0)), int(getattr(v, "align", 0)),
+            int(adjoint or getattr(v, "adjoint", 0) or 0), int(getattr(v, "binning", 0)),
+            int(getattr(v, "row0", 0)), int(getattr(v, "raster", 0)))
+
+
 def _struct_v(v, tile: int = 0, batch: int = 0, adjoint: int = 0) -> _abi.GsView:
-    tile = tile or getattr(v, "tile", 0) or 0
-    batch = batch or getattr(v, "batch", 0) or 0
-    adjoint = adjoint or getattr(v, "adjoint", 0) or 0
-    return _abi.GsView(int(v.lr_h), int(v.lr_w), int(v.out_h), int(v.out_w), float(v.scale),
-                       float(getattr(v, "trunc_k", 3.0)), int(getattr(v, "norm", 0)),
-                       int(tile), int(batch), int(getattr(v, "window", 0)),
-                       int(getattr(v, "align", 0)), int(adjoint), int(getattr(v, "binning", 0)),
-                       int(getattr(v, "row0", 0)), int(getattr(v, "raster", 0)))
+    return _abi.GsView(*_fields_v(v, tile, batch, adjoint))
 
 
 def _arrays(gs: Sequence[Gaussians], views, tile=0, batch=0):
+    """The checked ctypes arguments of one call. Built once per call and handed
+    to every library call it makes (sizing, count, render): building them costs
+    the host more than the calls themselves."""
     n = len(gs)
     if n != len(views) or n == 0:
         raise ValueError("need one view per image and at least one image")
-    structs = [_struct_g(g) for g in gs]
-    G = (_abi.GsGaussians * n)(*structs)
-    G._head_keep = [st._head_keep for st in structs]   # head structs the array points to
-    V = (_abi.GsView * n)(*[_struct_v(v, tile, batch) for v in views])
+    heads = {}   # one struct per head object of this call
+    for g in gs:
+        if g.head is not None and id(g.head) not in heads:
+            heads[id(g.head)] = _head_struct(g.head)
+    # (a ctypes array takes a tuple of fields per element)
+    G = (_abi.GsGaussians * n)(*[_fields_g(g, heads.get(id(g.head))) for g in gs])
+    G._head_keep = list(heads.values())   # head structs the array points to
+    V = (_abi.GsView * n)(*[_fields_v(v, tile, batch) for v in views])
     return n, G, V
 
 
@@ -187,12 +213,15 @@ class Workspace:
         return self.buf.numel()
 
 
-def workspace_bytes(gs, views, capacity: int, tile=0, batch=0) -> int:
-    n, G, V = _arrays(gs, views, tile, batch)
+def _ws_bytes(n, G, V, capacity: int) -> int:
     b = _abi.load().gs_workspace_size(n, G, V, int(capacity))
     if b == 0:
         raise _abi.GsError(_abi.GS_ERR_INVALID, "gs_workspace_size", _abi.last_error())
     return int(b)
+
+
+def workspace_bytes(gs, views, capacity: int, tile=0, batch=0) -> int:
+    return _ws_bytes(*_arrays(gs, views, tile, batch), capacity)
 
 
 def _check_ws(ws: Workspace, dev: torch.device):
@@ -200,23 +229,32 @@ def _check_ws(ws: Workspace, dev: torch.device):
         raise ValueError(f"workspace is on {ws.device}, the parameters on {dev}")
 
 
-def count_pairs(gs, views, tile=0, batch=0, stream=None) -> int:
-    """Exact number of (tile, Gaussian) pairs; synchronises the stream."""
-    n, G, V = _arrays(gs, views, tile, batch)
-    dev = _device(gs, stream)
-    ws = Workspace(workspace_bytes(gs, views, 0, tile, batch), dev)
+def _count(n, G, V, dev, stream) -> int:
+    ws = Workspace(_ws_bytes(n, G, V, 0), dev)
     out = ctypes.c_int64(0)
     _abi.check(_abi.load().gs_count_pairs(n, G, V, ws.ptr, ws.nbytes, _stream(stream),
                                           ctypes.byref(out)), "gs_count_pairs")
     return int(out.value)
 
 
+def count_pairs(gs, views, tile=0, batch=0, stream=None) -> int:
+    """Exact number of (tile, Gaussian) pairs; synchronises the stream."""
+    n, G, V = _arrays(gs, views, tile, batch)
+    return _count(n, G, V, _device(gs, stream), stream)
+
+
+def _new_workspace(n, G, V, dev, capacity=None, slack: float = 0.0, stream=None) -> Workspace:
+    if capacity is None:
+        capacity = _count(n, G, V, dev, stream)
+    capacity = int(capacity * (1.0 + slack)) + (1 if slack else 0)
+    return Workspace(_ws_bytes(n, G, V, capacity), dev)
+
+
 def make_workspace(gs, views, capacity=None, tile=0, batch=0, slack: float = 0.0,
                    stream=None) -> Workspace:
-    if capacity is None:
-        capacity = count_pairs(gs, views, tile, batch, stream)
-    capacity = int(capacity * (1.0 + slack)) + (1 if slack else 0)
-    return Workspace(workspace_bytes(gs, views, capacity, tile, batch), gs[0].rho.device)
+    n, G, V = _arrays(gs, views, tile, batch)
+    dev = _device(gs, stream) if capacity is None else gs[0].rho.device
+    return _new_workspace(n, G, V, dev, capacity, slack, stream)
 
 
 def render_batched(gs, views, outs=None, ws: Workspace | None = None, tile=0, batch=0,
@@ -226,12 +264,13 @@ def render_batched(gs, views, outs=None, ws: Workspace | None = None, tile=0, ba
     dev = _device(gs, stream)
     if outs is None:
         outs = [torch.empty((3, v.out_h, v.out_w), dtype=torch.float32, device=dev) for v in views]
-    if len(outs) != n:
-        raise ValueError("need one output per image")
-    for o, v in zip(outs, views):
-        _need(o, (3, v.out_h, v.out_w), torch.float32, dev, "output")
+    else:
+        if len(outs) != n:
+            raise ValueError("need one output per image")
+        for o, v in zip(outs, views):
+            _need(o, (3, v.out_h, v.out_w), torch.float32, dev, "output")
     if ws is None:
-        ws = make_workspace(gs, views, None, tile, batch, stream=stream)
+        ws = _new_workspace(n, G, V, dev, stream=stream)
     _check_ws(ws, dev)
     P = (ctypes.c_void_p * n)(*[o.data_ptr() for o in outs])
     _abi.check(_abi.load().gs_render_batched(n, G, V, P, ws.ptr, ws.nbytes, _stream(stream)),
@@ -254,10 +293,11 @@ def render_batched_bwd(gs, views, grad_outs, ws: Workspace, grads=None, tile=0, 
         _need(go, (3, v.out_h, v.out_w), torch.float32, dev, "grad_out")
     if grads is None:
         grads = [torch.empty((g.n, 9), dtype=torch.float32, device=dev) for g in gs]
-    if len(grads) != n:
-        raise ValueError("need one gradient buffer per image")
-    for gr, g in zip(grads, gs):
-        _need(gr, (g.n, 9), torch.float32, dev, "gradient buffer")
+    else:
+        if len(grads) != n:
+            raise ValueError("need one gradient buffer per image")
+        for gr, g in zip(grads, gs):
+            _need(gr, (g.n, 9), torch.float32, dev, "gradient buffer")
     GO = (ctypes.c_void_p * n)(*[g.data_ptr() for g in grad_outs])
     GR = (ctypes.c_void_p * n)(*[g.data_ptr() for g in grads])
     _abi.check(_abi.load().gs_render_batched_bwd(n, G, V, GO, GR, ws.ptr, ws.nbytes,
@@ -358,11 +398,9 @@ class GSRenderBatched(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, views, ref_grid_m, sizes, head, offset, sigma, rho, rgb, alpha):
-        gs, o = [], 0
-        ts = [t.contiguous() for t in (offset, sigma, rho, rgb, alpha)]
-        for n in sizes:
-            gs.append(Gaussians(*[t[o:o + n] for t in ts], ref_grid_m=ref_grid_m, head=head))
-            o += n
+        sizes, n = list(sizes), sum(sizes)
+        ts = [t.contiguous()[:n].split(sizes) for t in (offset, sigma, rho, rgb, alpha)]
+        gs = [Gaussians(*t, ref_grid_m=ref_grid_m, head=head) for t in zip(*ts)]
         outs, ws = render_batched(gs, views)
         ctx.gs, ctx.views, ctx.ws, ctx.dtype = gs, views, ws, offset.dtype
         return tuple(outs)
@@ -371,8 +409,9 @@ class GSRenderBatched(torch.autograd.Function):
     def backward(ctx, *grad_outs):
         go = [torch.zeros((3, v.out_h, v.out_w), device=ctx.gs[0].rho.device) if g is None else g
               for g, v in zip(grad_outs, ctx.views)]
-        grads = render_batched_bwd(ctx.gs, ctx.views, go, ctx.ws)
-        gr = torch.cat(grads, 0)
+        sizes = [g.n for g in ctx.gs]
+        gr = torch.empty((sum(sizes), 9), dtype=torch.float32, device=ctx.gs[0].rho.device)
+        render_batched_bwd(ctx.gs, ctx.views, go, ctx.ws, grads=gr.split(sizes))
         return (None, None, None, None, *_split_grads(gr, ctx.dtype))
 
 
@@ -389,7 +428,7 @@ class Plan:
         self.gs, self.views = list(gs), list(views)
         self.n, self.G, self.V = _arrays(self.gs, self.views, tile, batch)
         dev = _device(self.gs, stream)
-        self.ws = make_workspace(self.gs, self.views, capacity, tile, batch, slack, stream)
+        self.ws = _new_workspace(self.n, self.G, self.V, dev, capacity, slack, stream)
         self.outs = list(outs) if outs is not None else \
             [torch.empty((3, v.out_h, v.out_w), dtype=torch.float32, device=dev) for v in self.views]
         if len(self.outs) != self.n:
