@@ -99,8 +99,8 @@ typedef enum { GS_ALIGN_EQ4 = 0, GS_ALIGN_HALF = 1 } gs_align;
  *             atomics (summation order varies run to run);
  *   GAUSSIAN: one warp per Gaussian over its own window, one fixed summation
  *             order, no atomics: bitwise deterministic (when every image has
- *             ref_grid_m > 0 the warps work in CTAs over 8 x 8 blocks of LR
- *             cells, with the upstream gradient under the block staged in
+ *             ref_grid_m > 0 the warps work in CTAs over blocks of up to 8 x 8
+ *             LR cells, with the upstream gradient under the block staged in
  *             shared memory; the sums are the same);
  *   QUADRANT: TILE over the 8 x 8 quadrants of 16 x 16 tiles: a CTA per tile
  *             walks the (Gaussian, quadrant) pairs whose window meets the

@@ -234,8 +234,8 @@ __device__ __forceinline__ void cp_async16z(void* smem, const void* gmem, int sr
 }
 
 // Block form, for Gaussians on a reference grid (m > 0): one CTA per block of
-// kGbCellsX x kGbCellsY LR cells of an image. The CTA first forms the union box
-// of its Gaussians' windows and, when the box fits kGbFloats, copies the
+// gb_x x gb_y LR cells of an image (the host picks the shape: gblock_shape).
+// The CTA first forms the union box of its Gaussians' windows and, when the box fits kGbFloats, copies the
 // upstream gradient over it into shared memory once (three planes, the first
 // column even and the width even); its warps then walk their Gaussians (the
 // k-th of the block goes to warp k % kGbWarps) exactly as the one-warp form
@@ -260,16 +260,16 @@ __global__ void __launch_bounds__(kGbWarps * 32) k_raster_bwd_gblock(Ws w) {
   extern __shared__ float4 gstage4[];   // [3][RH][RW] floats (float4 for 16-byte alignment)
   float* gstage = reinterpret_cast<float*>(gstage4);
   __shared__ float4 rt[kGbWarps][kGwRows];
-  __shared__ float4 srec[kGbCellsX * kGbCellsY * kRecordF4];   // the records when m = 1
+  __shared__ float4 srec[kGbCells * kRecordF4];   // the records when m = 1
   __shared__ int sbox[4];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int im = image_of_gblock(w.images, w.n_images, (int)blockIdx.x);
   const ImageDesc& D = w.images[im];
-  const int bxs = (D.lr_w + kGbCellsX - 1) / kGbCellsX;
+  const int bxs = (D.lr_w + w.gb_x - 1) / w.gb_x;
   const int lb = (int)blockIdx.x - D.b_base;
   const int by = lb / bxs, bx = lb - by * bxs;
-  const int j0 = bx * kGbCellsX, i0 = by * kGbCellsY;
-  const int cw = min(kGbCellsX, D.lr_w - j0), ch = min(kGbCellsY, D.lr_h - i0);
+  const int j0 = bx * w.gb_x, i0 = by * w.gb_y;
+  const int cw = min(w.gb_x, D.lr_w - j0), ch = min(w.gb_y, D.lr_h - i0);
   const int m = D.m;
   const int ng = cw * ch * m;
   // global id of the block's k-th Gaussian (cells row by row, m per cell)

@@ -294,6 +294,29 @@ int team_of(const Problem& P, const gs_gaussians* g, const gs_view* v) {
   return P.tiles <= 304 ? 8 : 4;
 }
 
+// LR cells per block of the block Gaussian-warp adjoint. A block shares the
+// copied box of upstream gradient, so large blocks pay the windows' halo less
+// often, until the box no longer fits shared memory (then its Gaussians only
+// share L1) or the blocks are too few and too uneven to fill the chip. Measured,
+// us, 8 x 8 / 8 x 4 / 4 x 4 / 4 x 2 cells, one Gaussian per cell with sigma up to
+// 2: scale 4 75.6 / 81.2 / 97.5 / 127, 5 66.3 / 56.9 / 63.5 / 81.7, 6 68.5 / 60.8
+// / 51.3 / 62.1, 12 154 / 95.9 / 65.3 / 70.3; four per cell at scale 8 258 / 231
+// / 191 / 186; sixteen at scale 2 174 / 152 / 120 / 107; whole-image windows at
+// scale 3 569 / 291 / 162 / 160.
+void gblock_shape(int32_t n_images, const gs_gaussians* g, const gs_view* v, int32_t* x, int32_t* y) {
+  float scale = 0.0f;
+  int m = 0;
+  bool boxes = true;   // every window a k-sigma box
+  for (int i = 0; i < n_images; ++i) {
+    scale = std::max(scale, v[i].scale);
+    m = std::max(m, (int)g[i].ref_grid_m);
+    if (v[i].window != GS_WINDOW_SIGMA || !(v[i].trunc_k > 0.0f)) boxes = false;
+  }
+  const bool small = boxes && m <= 1;
+  *x = small && scale < 5.75f ? 8 : 4;
+  *y = small && scale < 4.5f ? 8 : m >= 16 ? 2 : 4;
+}
+
 struct Call {
   Problem P;
   Layout L;
@@ -357,11 +380,12 @@ gs_status prepare(int32_t n_images, const gs_gaussians* g, const gs_view* v, voi
   w.adjoint = c->P.adjoint;
   // blocks of LR cells (the Gaussian-warp adjoint's block form), when
   // every image's Gaussians sit on a reference grid
+  gblock_shape(n_images, g, v, &w.gb_x, &w.gb_y);
   int64_t gblocks = 0;
   for (int i = 0; i < n_images; ++i) {
     if (g[i].ref_grid_m == 0) { gblocks = 0; break; }
-    gblocks += (int64_t)((v[i].lr_h + kGbCellsY - 1) / kGbCellsY) *
-               ((v[i].lr_w + kGbCellsX - 1) / kGbCellsX);
+    gblocks += (int64_t)((v[i].lr_h + w.gb_y - 1) / w.gb_y) *
+               ((v[i].lr_w + w.gb_x - 1) / w.gb_x);
   }
   w.n_gblocks = gblocks < (1LL << 31) ? (int32_t)gblocks : 0;
   return GS_OK;
@@ -419,7 +443,7 @@ gs_status upload_images(const Call& c, const gs_gaussians* g, const gs_view* v, 
       d.p_base = pbase;
       d.b_base = bbase;
       gbase += g[i].n;
-      bbase += ((v[i].lr_h + kGbCellsY - 1) / kGbCellsY) * ((v[i].lr_w + kGbCellsX - 1) / kGbCellsX);
+      bbase += ((v[i].lr_h + c.w.gb_y - 1) / c.w.gb_y) * ((v[i].lr_w + c.w.gb_x - 1) / c.w.gb_x);
       tbase += d.tiles_x * d.tiles_y;
       pbase += d.tiles_y * ((d.tiles_x + 1) / 2);
     }

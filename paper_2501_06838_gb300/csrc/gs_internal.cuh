@@ -15,8 +15,7 @@ enum : uint32_t { kStInvalid = 1u, kStCapacity = 2u, kStInternal = 4u, kStTimeou
 constexpr int kSetupChunk = 16;       // image descriptors per setup launch
 constexpr int kFootprintBlock = 256;  // Gaussians per footprint / emit block
 constexpr int kRecordF4 = 4;          // a record is 4 float4 = 64 B
-constexpr int kGbCellsX = 8;          // LR cells per block of the block Gaussian-warp adjoint
-constexpr int kGbCellsY = 8;
+constexpr int kGbCells = 64;          // LR cells at most per block of the block Gaussian-warp adjoint
 
 // Per-image descriptor, copied into the workspace at the start of each call.
 struct ImageDesc {
@@ -115,6 +114,7 @@ struct Ws {
   int32_t adjoint;            // the adjoint kernel of these views (gs_adjoint, resolved)
   int32_t bwd_parts;          // tile and quadrant adjoints: parts of each tile's list
   int32_t n_gblocks;          // every image with m > 0: blocks of LR cells in all; else 0
+  int32_t gb_x, gb_y;         // cells per block
   const float* grad_out0;     // direct: dL/dI of image 0
   float* grads0;              // direct: parameter gradients of image 0
 };
