@@ -107,9 +107,9 @@ typedef enum { GS_ALIGN_EQ4 = 0, GS_ALIGN_HALF = 1 } gs_align;
  *             quadrant, so small windows waste fewer pixel evaluations at tile
  *             edges. Needs tile 16 (GS_ERR_UNSUPPORTED otherwise);
  *   AUTO:     QUADRANT at tile 16 when every view uses the SIGMA window with
- *             trunc_k > 0 and every scale is < 10 or the images have fewer
- *             than 3 Gaussians per tile (small windows, or short lists, where
- *             it measured faster), else TILE
+ *             trunc_k > 0 and every scale is < 10, or < 14 with fewer than 3
+ *             Gaussians per tile (small windows, or short lists, where it
+ *             measured faster and no less exact), else TILE
  *             (GAUSSIAN re-reads grad_out once per (Gaussian, pixel) pair
  *             instead of once per (tile, pixel) and measured slower).
  * All compute the same derivative (Eq. 4 with the windows held fixed). */

@@ -138,7 +138,8 @@ gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Pr
   P->tile = tile_of(v[0]);
   P->batch = batch_of(v[0]);
   bool grid_ok = true;   // every image on a reference grid, coordinates fit int16
-  bool sigma_windows = true, large_scale = false, larger_scale = false;   // for AUTO (>= 6, >= 10)
+  bool sigma_windows = true;   // for the AUTO raster layout and adjoint
+  float max_scale = 0.0f;
   bool truncated = true;                             // every window a k-sigma box (trunc_k > 0)
   for (int i = 0; i < n_images; ++i) {
     const gs_gaussians& G = g[i];
@@ -170,8 +171,7 @@ gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Pr
     if (V.raster != v[0].raster)
       return fail(GS_ERR_INVALID, "image %lld: raster differs from image 0", (long long)i);
     if (V.window != GS_WINDOW_SIGMA) sigma_windows = false;
-    if (V.scale >= 6.0f) large_scale = true;
-    if (V.scale >= 10.0f) larger_scale = true;
+    max_scale = std::max(max_scale, V.scale);
     if (!(V.trunc_k > 0.0f)) truncated = false;
     if (G.ref_grid_m == 0 || V.out_w > 32767 || V.out_h > 32767) grid_ok = false;
     const double sh = std::floor((double)V.scale * V.lr_h) + 1.0;
@@ -218,19 +218,21 @@ gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Pr
   if (v[0].raster == GS_RASTER_PAIR && !pair_ok)
     return fail(GS_ERR_UNSUPPORTED, "raster PAIR needs grid binning and tile 16");
   P->pair = (v[0].raster == GS_RASTER_PAIR ||
-             (v[0].raster == GS_RASTER_AUTO && pair_ok && sigma_windows && large_scale)) ? 1 : 0;
+             (v[0].raster == GS_RASTER_AUTO && pair_ok && sigma_windows && max_scale >= 6.0f)) ? 1 : 0;
   if (v[0].adjoint == GS_ADJOINT_QUADRANT && P->tile != 16)
     return fail(GS_ERR_UNSUPPORTED, "adjoint QUADRANT needs tile 16");
   // AUTO: quadrants at tile 16 where every view has truncated SIGMA windows and
-  // the windows are small (every scale < 10) or the lists short (fewer than 3
-  // Gaussians per tile): whole tiles waste less with large windows and full
-  // chunks. Measured, whole tiles against quadrants, 4 Gaussians per LR pixel
-  // with sigma up to 3: scale 8 1030 against 993 us, 10 716 against 705, 12
-  // 941 against 979; 1 Gaussian per LR pixel with sigma up to 2: scale 6 62.8
-  // against 50.1, 12 510 against 463, 16 372 against 332; 12,288 Gaussians at
-  // scale 24 142 against 139.
+  // the windows are small (every scale < 10) or not too large with short lists
+  // (scale < 14, fewer than 3 Gaussians per tile): whole tiles waste less with
+  // large windows and full chunks. Measured, us, whole tiles against quadrants,
+  // 4 Gaussians per LR pixel with sigma up to 3: scale 8 1030 against 993, 10
+  // 716 against 705, 12 941 against 979; 1 Gaussian per LR pixel with sigma up
+  // to 2: scale 6 62.8 against 50.1, 12 510 against 463. The gradients' error
+  // against 64 bits is smaller with quadrants up to there (scale 6 2.5e-7
+  // against 3.2e-7, 12 2.7e-7 against 3.0e-7), larger beyond, where a window
+  // adds the sums of hundreds of quadrants (scale 24 3.8e-7 against 2.8e-7).
   const bool quad_auto = P->tile == 16 && sigma_windows && truncated &&
-                         (!larger_scale || P->n < 3 * P->tiles);
+                         (max_scale < 10.0f || (max_scale < 14.0f && P->n < 3 * P->tiles));
   P->adjoint = v[0].adjoint == GS_ADJOINT_GAUSSIAN ? GS_ADJOINT_GAUSSIAN
                : (v[0].adjoint == GS_ADJOINT_QUADRANT ||
                   (v[0].adjoint == GS_ADJOINT_AUTO && quad_auto)) ? GS_ADJOINT_QUADRANT
