@@ -232,7 +232,7 @@ size_t gs_workspace_size(int32_t n_images, const gs_gaussians* g, const gs_view*
                          int64_t pair_capacity);
 
 /* Exact number of (tile, Gaussian) pairs the render of these images emits.
- * Runs the per-Gaussian footprint pass and the prefix sum on `stream` inside
+ * Runs a counting pass over the Gaussians' windows on `stream` inside
  * `ws` (which needs capacity >= 0 only), then SYNCHRONISES the stream and
  * writes the count to *pairs_out (host pointer). Device status problems are
  * returned directly. */

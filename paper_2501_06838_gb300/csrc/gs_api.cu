@@ -640,15 +640,11 @@ gs_status gs_count_pairs(int32_t n_images, const gs_gaussians* g, const gs_view*
   Call c;
   gs_status st = prepare(n_images, g, v, ws, ws_bytes, &c);
   if (st != GS_OK) return st;
+  c.w.grid = 0;   // the count is the same either way, and needs no per-tile counts
   st = upload_images(c, g, v, nullptr, nullptr, nullptr, 1, s);
   if (st != GS_OK) return st;
-  c.w.grid = 0;   // the count is the same either way; take it from the scan
-  cudaError_t e = launch_preprocess(c.w, s);
-  if (e != cudaSuccess) return cuda_fail(e, "preprocess");
-  if (c.w.n > 0) {
-    e = launch_scan_counts(c.w, s);
-    if (e != cudaSuccess) return cuda_fail(e, "scan");
-  }
+  cudaError_t e = launch_count(c.w, s);
+  if (e != cudaSuccess) return cuda_fail(e, "count");
   Header h;
   e = cudaMemcpyAsync(&h, c.w.hdr, sizeof(Header), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

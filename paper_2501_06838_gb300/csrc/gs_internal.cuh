@@ -61,7 +61,7 @@ struct Header {
   unsigned long long pairs;        // P, total (tile, Gaussian) pairs
   unsigned long long pixel_pairs;  // sum_i |R_i|
   unsigned long long capacity;
-  uint32_t work_counter;            // next tile (or pair) for the forward raster's CTAs
+  uint32_t work_counter;            // blocks of the count pass that are done
   uint32_t bwd_counter;             // next tile for the tile adjoint's CTAs
   unsigned long long list_cursor;  // grid mode: pair-list slots handed out to tiles
   unsigned long long reserved[10];
@@ -225,6 +225,7 @@ __device__ __forceinline__ unsigned long long effective_pairs(const Header* h) {
 // ---------------------------------------------------------------------------
 cudaError_t launch_setup(const SetupChunk& c, const Ws& w, cudaStream_t s);
 cudaError_t launch_preprocess(const Ws& w, cudaStream_t s);
+cudaError_t launch_count(const Ws& w, cudaStream_t s);   // pairs, window areas and status only
 cudaError_t launch_preprocess_bwd(const Ws& w, cudaStream_t s);
 cudaError_t launch_scan_counts(const Ws& w, cudaStream_t s);
 cudaError_t launch_emit(const Ws& w, cudaStream_t s);
