@@ -480,8 +480,6 @@ gs_status run_forward(int32_t n_images, const gs_gaussians* g, const gs_view* v,
   e = launch_preprocess(c.w, s);
   if (e != cudaSuccess) return cuda_fail(e, "preprocess");
   if (c.w.n > 0) {
-    e = launch_scan_counts(c.w, s);
-    if (e != cudaSuccess) return cuda_fail(e, "scan");
     e = launch_emit(c.w, s);
     if (e != cudaSuccess) return cuda_fail(e, "emit");
   }

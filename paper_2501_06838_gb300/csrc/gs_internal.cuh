@@ -227,7 +227,6 @@ cudaError_t launch_setup(const SetupChunk& c, const Ws& w, cudaStream_t s);
 cudaError_t launch_preprocess(const Ws& w, cudaStream_t s);
 cudaError_t launch_count(const Ws& w, cudaStream_t s);   // pairs, window areas and status only
 cudaError_t launch_preprocess_bwd(const Ws& w, cudaStream_t s);
-cudaError_t launch_scan_counts(const Ws& w, cudaStream_t s);
 cudaError_t launch_emit(const Ws& w, cudaStream_t s);
 cudaError_t launch_sort(const Ws& w, int key_bits, cudaStream_t s, int* final_buf);
 cudaError_t launch_ranges(const Ws& w, const uint32_t* sorted_keys, cudaStream_t s);
