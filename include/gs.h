@@ -146,8 +146,9 @@ typedef enum { GS_BINNING_AUTO = 0, GS_BINNING_SORT = 1, GS_BINNING_GRID = 2 } g
  *         loads) is shared by the two tiles. Needs GRID binning and tile 16
  *         (GS_ERR_UNSUPPORTED otherwise);
  *   AUTO: PAIR with GRID binning at tile 16 when every view uses the SIGMA
- *         window and some view's scale is >= 6 (large windows, where it
- *         measured faster), else TILE. */
+ *         window and the pairs are enough to fill the chip with short lists
+ *         (where it measured faster: some scale >= 4 and 5,000 pairs, >= 10 and
+ *         1,200 pairs, or >= 6 and fewer than 256), else TILE. */
 typedef enum { GS_RASTER_AUTO = 0, GS_RASTER_TILE = 1, GS_RASTER_PAIR = 2 } gs_raster;
 
 /* The Gaussian primary head's activations (Sec. 3.2, "Gaussian Primary Head"),

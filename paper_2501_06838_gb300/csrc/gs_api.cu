@@ -123,11 +123,28 @@ struct Problem {
   int n_images;
   int64_t n;
   int64_t tiles;
+  int64_t tile_pairs;   // horizontal pairs of tiles
   int tile, batch;
   int adjoint;   // gs_adjoint resolved: 1 tile, 2 Gaussian-warp, 3 tile quadrants
   int grid;      // gs_binning resolved: 1 grid-implicit, 0 sorted pair list
   int pair;      // gs_raster resolved: 1 one warp per pair of tiles, 0 per tile
 };
+
+// Whether the forward over pairs of tiles pays (AUTO, k-sigma windows). A pair
+// shares staging and steps between two tiles but makes half as many and twice
+// as long warps, 16 per SM instead of 21, so the pairs have to fill the chip a
+// few times over, and the longer the lists, the more times. Measured, us, tiles /
+// pairs: 1 Gaussian per LR pixel at scale 5, 1,250 pairs 21.5 / 22.6, 6,441 67.6
+// / 65.9, 13,366 128 / 121; at scale 12, 2,850 pairs 29.2 / 27.9, 13,366 96.8 /
+// 84.2; 4 per pixel (sigma up to 3) at scale 8, 2,850 pairs 125 / 138, 6,441 255
+// / 244, at scale 4, 13,366 pairs 690 / 727; 16 per pixel at scale 8, 6,441 pairs
+// 677 / 730. Below 256 pairs either layout is one short round of warps on part of
+// the chip (tiles 12 to 14 us, pairs 13 to 16): the large scales keep pairs.
+bool pairs_pay(int64_t pairs, int64_t n, int64_t tiles, float scale) {
+  if (scale >= 4.0f && pairs >= 5000) return n < (scale >= 6.0f ? 30 : 18) * tiles;
+  if (scale >= 10.0f && pairs >= 1200) return n < 8 * tiles;
+  return scale >= 6.0f && pairs < 256 && n < 8 * tiles;
+}
 
 gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Problem* P) {
   if (n_images < 1) return fail(GS_ERR_INVALID, "n_images must be >= 1 (got %lld)", (long long)n_images);
@@ -135,6 +152,7 @@ gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Pr
   P->n_images = n_images;
   P->n = 0;
   P->tiles = 0;
+  P->tile_pairs = 0;
   P->tile = tile_of(v[0]);
   P->batch = batch_of(v[0]);
   bool grid_ok = true;   // every image on a reference grid, coordinates fit int16
@@ -197,6 +215,7 @@ gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Pr
     const int64_t tx = (V.out_w + t - 1) / t, ty = (V.out_h + t - 1) / t;
     P->n += G.n;
     P->tiles += tx * ty;
+    P->tile_pairs += (tx + 1) / 2 * ty;
   }
   if (!(P->tile == 8 || P->tile == 16 || P->tile == 32))
     return fail(GS_ERR_INVALID, "tile must be 8, 16 or 32 (got %lld)", (long long)P->tile);
@@ -218,7 +237,8 @@ gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Pr
   if (v[0].raster == GS_RASTER_PAIR && !pair_ok)
     return fail(GS_ERR_UNSUPPORTED, "raster PAIR needs grid binning and tile 16");
   P->pair = (v[0].raster == GS_RASTER_PAIR ||
-             (v[0].raster == GS_RASTER_AUTO && pair_ok && sigma_windows && max_scale >= 6.0f)) ? 1 : 0;
+             (v[0].raster == GS_RASTER_AUTO && pair_ok && sigma_windows &&
+              pairs_pay(P->tile_pairs, P->n, P->tiles, max_scale))) ? 1 : 0;
   if (v[0].adjoint == GS_ADJOINT_QUADRANT && P->tile != 16)
     return fail(GS_ERR_UNSUPPORTED, "adjoint QUADRANT needs tile 16");
   // AUTO: quadrants at tile 16 where every view has truncated SIGMA windows and
