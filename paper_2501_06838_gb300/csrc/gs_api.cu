@@ -283,15 +283,18 @@ int radix_passes(int64_t tiles) { return (key_bits(tiles) + 8) / 9; }
 
 // Warps per tile of the tile-16 forward: a team where lists are long (0: one
 // warp). A list's segments of 512 entries are what a team shares, so the rule
-// asks for lists of some segments: known from the views with the ratio window
-// (and the whole image, trunc_k <= 0); with k-sigma boxes only bounded below by
-// the Gaussians per tile, and then only where the tiles are few enough for all
-// teams to be resident at once (2 of 8 warps or 5 of 4 per SM, 152 SMs), where
-// idle warps take nobody's place. Measured, one warp -> team: 2,025 tiles with
-// lists of 23,000 3.73 -> 2.99 ms (8 warps: 3.11), 8,100 tiles with 6,400 3.08
-// -> 2.94 ms, 2,025 tiles with 1,500 320 -> 263 us, 250 tiles with 4,000 to
-// 10,000 547 -> 117 us (4 warps: 154), 256 tiles with 16 Gaussians per LR pixel
-// 115 -> 54 us; 625 tiles with lists of 80 14.2 -> 16.1 us, so those keep one.
+// asks for lists of some segments. Their length is known from the views with
+// the ratio window (and the whole image, trunc_k <= 0); with k-sigma boxes it is
+// bounded below by the Gaussians per tile (lists are 3 to 9 times that). Where
+// the tiles are few enough for all teams to be resident at once (2 of 8 warps or
+// 5 of 4 per SM, 152 SMs) idle warps take nobody's place, and building the list
+// together pays already. Measured, one warp -> team: ratio window, 2,025 tiles
+// with lists of 23,000 3.73 -> 2.99 ms (8 warps: 3.11), 8,100 tiles with 6,400
+// 3.08 -> 2.94 ms, 2,025 tiles with 1,500 320 -> 263 us, 250 tiles with 4,000 to
+// 10,000 547 -> 117 us (4 warps: 154); boxes, us, at 100 to 729 tiles: 96
+// Gaussians per tile 86.8 -> 40.6, 64 77.8 -> 48.7, 24 34.9 -> 28.9, 16 no change;
+// at 3,249 tiles: 643 516 -> 431, 251 331 -> 306, 140 183 -> 211; at 15,625 tiles:
+// 655 2000 -> 1973, 455 1014 -> 1127.
 int team_of(const Problem& P, const gs_gaussians* g, const gs_view* v) {
   if (P.tile != 16 || P.pair || P.batch == 64) return 0;
   double listed = 0.0;
@@ -312,7 +315,8 @@ int team_of(const Problem& P, const gs_gaussians* g, const gs_view* v) {
   }
   listed /= (double)P.tiles;
   const bool few = P.tiles <= 760;
-  if (!(known ? listed >= (few ? 512.0 : 1024.0) : few && listed >= 128.0)) return 0;
+  const double line = known ? (few ? 512.0 : 1024.0) : few ? 20.0 : P.tiles <= 3300 ? 240.0 : 600.0;
+  if (listed < line) return 0;
   return P.tiles <= 304 ? 8 : 4;
 }
 
