@@ -503,66 +503,111 @@ __device__ __forceinline__ void issue_slots(const Ws& w, const uint32_t (&ids)[P
   cp_async_commit();
 }
 
-// Writes a lane's pixels: columns x .., rows y and y + 1 of the output.
+// The region's pixels through shared memory, for stores in whole rows: 128-byte
+// lines of a row (NQ 2) or a row pair (NQ 1), their 16-byte pieces permuted by
+// the row pair so that neither side has bank conflicts.
 template <int NQ>
-__device__ __forceinline__ void store_strips(const ImageDesc* D, const StripAcc<NQ>& acc, int x,
-                                             int y) {
+__device__ __forceinline__ void strips_to_rows(const StripAcc<NQ>& acc, float* buf, int lane) {
+  const int strip = lane >> 3, rp = lane & 7;
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int h = 0; h < NQ; ++h)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int line = NQ == 2 ? 2 * rp + j : rp, piece = NQ == 2 ? 2 * strip + h : 4 * j + strip;
+        const float2 a = acc[j][2 * h][k], b = acc[j][2 * h + 1][k];
+        *reinterpret_cast<float4*>(buf + k * 256 * NQ + line * 32 + 4 * (piece ^ rp)) =
+            make_float4(a.x, a.y, b.x, b.y);
+      }
+}
+// Column lane % (16 NQ) of row r of channel k.
+template <int NQ>
+__device__ __forceinline__ float row_value(const float* buf, int k, int r, int lane) {
+  return buf[k * 256 * NQ + (NQ == 2 ? r : r >> 1) * 32 + 4 * ((lane >> 2) ^ (r >> 1)) + (lane & 3)];
+}
+
+// Writes the region's pixels: 16 NQ columns from ox, 16 rows from output row y0.
+// A pair of tiles goes out in whole rows by way of the table's memory: stored by
+// their lanes, 16 bytes or (rows not 16-byte aligned) 4 at a time, its pixels
+// were parts of 32-byte sectors (16 images of odd widths, 630 MB, with all but
+// the stores left out: 2 TB/s; in all 760 -> 702 us; 915 -> 912 us at 5760 x
+// 3240). One tile's lanes store their own: a store has four whole strips in a
+// row, and the way through shared memory took as long (1002 x 751: 50.6 us both,
+// 16 crops 37.3 against 36.4).
+template <int NQ>
+__device__ __forceinline__ void store_strips(const ImageDesc* D, const StripAcc<NQ>& acc,
+                                             StripTables<NQ>& t, int ox, int y0) {
+  const int lane = threadIdx.x & 31, strip = lane >> 3, rp = lane & 7;
   const int H = D->out_h, W = D->out_w;
   float* out = D->out;
   const int64_t plane = (int64_t)H * W;
   // four columns per store where the output's rows are 16-byte aligned
   const bool vec = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+  if constexpr (NQ == 1) {
+    const int x = ox + 4 * strip, y = y0 + 2 * rp;
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    if (y + j >= H) continue;
-#pragma unroll
-    for (int h = 0; h < NQ; ++h) {
-      const int xh = x + 4 * h;
-      if (xh >= W) continue;
+    for (int j = 0; j < 2; ++j) {
+      if (y + j >= H || x >= W) continue;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        float* o = out + k * plane + (int64_t)(y + j) * W + xh;
-        const float2 a = acc[j][2 * h][k], b = acc[j][2 * h + 1][k];
+        float* o = out + k * plane + (int64_t)(y + j) * W + x;
+        const float2 a = acc[j][0][k], b = acc[j][1][k];
         if (vec) {
           *reinterpret_cast<float4*>(o) = make_float4(a.x, a.y, b.x, b.y);
         } else {
           o[0] = a.x;
-          if (xh + 1 < W) o[1] = a.y;
-          if (xh + 2 < W) o[2] = b.x;
-          if (xh + 3 < W) o[3] = b.y;
+          if (x + 1 < W) o[1] = a.y;
+          if (x + 2 < W) o[2] = b.x;
+          if (x + 3 < W) o[3] = b.y;
         }
       }
+    }
+  } else {
+    float* buf = reinterpret_cast<float*>(&t);
+    strips_to_rows<NQ>(acc, buf, lane);
+    __syncwarp();
+    if (vec) {
+      const int piece = lane & 7, r0 = lane >> 3, x = ox + 4 * piece;
+      const int rows = x < W ? H - y0 - r0 : 0;   // of this lane, from its first
+      float* o = out + (int64_t)(y0 + r0) * W + x;
+#pragma unroll
+      for (int k = 0; k < 3; ++k, o += plane)
+#pragma unroll
+        for (int i = 0; i < 16; i += 4)
+          if (i < rows)
+            *reinterpret_cast<float4*>(o + (int64_t)i * W) = *reinterpret_cast<const float4*>(
+                buf + k * 512 + (r0 + i) * 32 + 4 * (piece ^ ((r0 + i) >> 1)));
+    } else {
+      const int x = ox + lane;
+      const int rows = x < W ? H - y0 : 0;
+      float* o = out + (int64_t)y0 * W + x;
+#pragma unroll
+      for (int k = 0; k < 3; ++k, o += plane)
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (i < rows) o[(int64_t)i * W] = row_value<NQ>(buf, k, i, lane);
     }
   }
 }
 
-// A segment's end (rare: its code is kept small): puts the region's pixels (16
-// NQ columns from ox, 16 rows from output row y0) through the table's shared
-// memory onto the output and clears them. go / add, the same over a tile's
-// lanes: whether the lane's tile is written, and whether onto what an earlier
-// segment left. (Every tile's last store taking this way as well cost 4% to 8%
-// of the forward.)
+// A segment's end (rare: its code is kept small): puts the region's pixels onto
+// the output and clears them. go / add, the same over a tile's lanes: whether
+// the lane's tile is written, and whether onto what an earlier segment left.
 template <int NQ>
 __device__ __forceinline__ void fold_strips(const ImageDesc* D, StripAcc<NQ>& acc,
                                             StripTables<NQ>& t, int ox, int y0, bool go, bool add) {
-  constexpr int C = 16 * NQ, PLANE = 16 * C;
-  static_assert(sizeof(t.x) + sizeof(t.r) >= 3 * PLANE * sizeof(float), "the sums fit the table");
-  const int lane = threadIdx.x & 31, strip = lane >> 3, rp = lane & 7;
+  constexpr int C = 16 * NQ;
+  static_assert(sizeof(t.x) + sizeof(t.r) >= 48 * C * sizeof(float), "the sums fit the table");
+  const int lane = threadIdx.x & 31;
   float* buf = reinterpret_cast<float*>(&t);
   __syncwarp();
   if (go) {
+    strips_to_rows<NQ>(acc, buf, lane);
 #pragma unroll
     for (int j = 0; j < 2; ++j)
 #pragma unroll
-      for (int h = 0; h < NQ; ++h)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          float2& a = acc[j][2 * h][k];
-          float2& b = acc[j][2 * h + 1][k];
-          *reinterpret_cast<float4*>(buf + k * PLANE + (2 * rp + j) * C + 4 * (NQ * strip + h)) =
-              make_float4(a.x, a.y, b.x, b.y);
-          a = b = f2(0.0f, 0.0f);
-        }
+      for (int h = 0; h < 2 * NQ; ++h) acc[j][h][0] = acc[j][h][1] = acc[j][h][2] = f2(0.0f, 0.0f);
   }
   __syncwarp();
   const int H = D->out_h, W = D->out_w;
@@ -574,7 +619,7 @@ __device__ __forceinline__ void fold_strips(const ImageDesc* D, StripAcc<NQ>& ac
 #pragma unroll 4
       for (int r = lane / C; r < 16; r += 32 / C) {
         if (y0 + r >= H) break;
-        const float v = buf[k * PLANE + r * C + lane % C];
+        const float v = row_value<NQ>(buf, k, r, lane);
         o[(int64_t)r * W] = add ? o[(int64_t)r * W] + v : v;
       }
     }
@@ -689,7 +734,7 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
   if (total > kSeg)
     fold_strips<1>(D, acc, T[0], ox, oy - D->row0, true, true);
   else
-    store_strips<1>(D, acc, ox + 4 * strip, oy - D->row0 + 2 * rp);
+    store_strips<1>(D, acc, T[0], ox, oy - D->row0);
 }
 
 // ---------------------------------------------------------------------------
@@ -1255,7 +1300,7 @@ __global__ void __launch_bounds__(32, 16) k_raster_fwd_pair(Ws w) {
   if (written_a + written_b > 0)
     fold_strips<2>(D, acc, T[0], ox, oy - D->row0, true, (strip < 2 ? written_a : written_b) > 0);
   else
-    store_strips<2>(D, acc, ox + 8 * strip, oy - D->row0 + 2 * rp);
+    store_strips<2>(D, acc, T[0], ox, oy - D->row0);
 }
 
 template <int TILE, int BY, int PF>

@@ -45,3 +45,25 @@ def test_strip_columns_and_stores(w, offset):
     ref = oracle.render(g, v)
     assert np.all(normwise(out.cpu().double().numpy(), ref, axis=(1, 2)) < 1e-5)
     assert torch.all(buf[:offset] == -7.0) and torch.all(buf[offset + 3 * h * w:] == -7.0)
+
+
+@pytest.mark.parametrize("w", [1, 4, 15, 16, 17, 20, 31, 32, 33, 47, 48, 50, 64])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_pair_stores(w, offset):
+    """Pairs of tiles go out in rows: the one-tile layout's bits, and nothing
+    outside the image."""
+    import torch
+    import paper_2501_06838_gb300 as gs
+    h = 21
+    g = S.draw_gaussians(w, h, w, 4, (0.2, 2.0))
+    v = S.View(h, w, h, w, 1.0)
+    dg = device_gaussians(g)
+    v.binning, v.raster = 2, 1
+    want, _ = gs.render(dg, v, check=True)
+    buf = torch.full((offset + 3 * h * w + 8,), -7.0, device="cuda")
+    out = buf[offset:offset + 3 * h * w].view(3, h, w)
+    v.raster = 2
+    _, ws = gs.render(dg, v, out=out, check=True)
+    assert gs.read_stats(ws)["raster"] == 2
+    assert torch.equal(out, want)
+    assert torch.all(buf[:offset] == -7.0) and torch.all(buf[offset + 3 * h * w:] == -7.0)
