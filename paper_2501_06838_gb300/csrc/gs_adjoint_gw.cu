@@ -189,8 +189,7 @@ __device__ __forceinline__ void gw_walk(const float* __restrict__ go, int64_t pl
 }
 
 __global__ void __launch_bounds__(kGwWarps * 32) k_raster_bwd_gw(Ws w) {
-  griddep_release();
-  griddep_wait();
+  griddep_enter(w);
   __shared__ float4 rt[kGwWarps][kGwRows];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int64_t gi = (int64_t)blockIdx.x * kGwWarps + wp;
@@ -255,8 +254,7 @@ __device__ __forceinline__ int image_of_gblock(const ImageDesc* im, int n_images
 }
 
 __global__ void __launch_bounds__(kGbWarps * 32) k_raster_bwd_gblock(Ws w) {
-  griddep_release();
-  griddep_wait();
+  griddep_enter(w);
   extern __shared__ float4 gstage4[];   // [3][RH][RW] floats (float4 for 16-byte alignment)
   float* gstage = reinterpret_cast<float*>(gstage4);
   __shared__ float4 rt[kGbWarps][kGwRows];

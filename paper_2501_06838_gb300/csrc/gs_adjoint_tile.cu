@@ -321,8 +321,7 @@ __device__ __forceinline__ void bwd_block(const Ws& w, const BlockSmem& S, int e
 
 template <bool SPLIT>
 __global__ void __launch_bounds__(32 * kBwWarps) k_raster_bwd_quad(Ws w, const uint32_t* vals) {
-  griddep_release();
-  griddep_wait();
+  griddep_enter(w);
   constexpr int NT = 32 * kBwWarps;
   __shared__ BlockSmem S;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -412,8 +411,7 @@ __global__ void __launch_bounds__(32 * kBwWarps) k_raster_bwd_quad(Ws w, const u
 // at 64 for 32 resident CTAs per SM (no spills at tile 8, 16 or 32).
 template <int TILE, bool SPLIT>
 __global__ void __launch_bounds__(32, 32) k_raster_bwd_tile(Ws w, const uint32_t* vals) {
-  griddep_release();
-  griddep_wait();
+  griddep_enter(w);
   __shared__ float4 sgA[TILE * TILE / 2];
   __shared__ float2 sgB[TILE * TILE / 2];
   const uint32_t parts = SPLIT ? (uint32_t)w.bwd_parts : 1u, units = (uint32_t)w.tiles * parts;

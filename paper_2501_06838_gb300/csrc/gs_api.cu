@@ -417,6 +417,41 @@ gs_status prepare(int32_t n_images, const gs_gaussians* g, const gs_view* v, voi
   return GS_OK;
 }
 
+// An image's descriptor as the first of a batch; no outputs or gradients.
+ImageDesc describe(const gs_gaussians& G, const gs_view& V, int tile) {
+  ImageDesc d;
+  std::memset(&d, 0, sizeof(d));
+  d.off = G.offset;
+  d.sig = G.sigma;
+  d.rho = G.rho;
+  d.rgb = G.rgb;
+  d.alpha = G.alpha;
+  d.n = G.n;
+  d.dtype = G.dtype;
+  d.m = G.ref_grid_m;
+  d.lr_h = V.lr_h;
+  d.lr_w = V.lr_w;
+  d.out_h = V.out_h;
+  d.out_w = V.out_w;
+  d.row0 = V.row0;
+  d.scale = V.scale;
+  d.trunc_k = V.trunc_k;
+  d.flags = (V.norm == GS_NORM_PEAK ? kFlagPeak : 0) |
+            (V.window == GS_WINDOW_RATIO ? kFlagRatio : 0) |
+            (V.align == GS_ALIGN_HALF ? kFlagHalf : 0) |
+            (G.head ? kFlagHead : 0) |
+            (G.head && G.head->offset_tanh ? kFlagOffsetTanh : 0);
+  if (G.head) {
+    d.h_sigma_lo = G.head->sigma_lo;
+    d.h_sigma_span = G.head->sigma_span;
+    d.h_rho_scale = G.head->rho_scale;
+    d.h_offset_scale = G.head->offset_scale;
+  }
+  d.tiles_x = (V.out_w + tile - 1) / tile;
+  d.tiles_y = (V.out_h + tile - 1) / tile;
+  return d;
+}
+
 gs_status upload_images(const Call& c, const gs_gaussians* g, const gs_view* v, float* const* outs,
                         const float* const* grad_outs, float* const* grads, int reset,
                         cudaStream_t s) {
@@ -433,38 +468,11 @@ gs_status upload_images(const Call& c, const gs_gaussians* g, const gs_view* v, 
     for (int k = 0; k < ch.count; ++k) {
       const int i = first + k;
       ImageDesc& d = ch.d[k];
-      d.off = g[i].offset;
-      d.sig = g[i].sigma;
-      d.rho = g[i].rho;
-      d.rgb = g[i].rgb;
-      d.alpha = g[i].alpha;
+      d = describe(g[i], v[i], tile);
       d.out = outs ? outs[i] : nullptr;
       d.grad_out = grad_outs ? grad_outs[i] : nullptr;
       d.grads = grads ? grads[i] : nullptr;
-      d.n = g[i].n;
       d.g_base = gbase;
-      d.dtype = g[i].dtype;
-      d.m = g[i].ref_grid_m;
-      d.lr_h = v[i].lr_h;
-      d.lr_w = v[i].lr_w;
-      d.out_h = v[i].out_h;
-      d.out_w = v[i].out_w;
-      d.row0 = v[i].row0;
-      d.scale = v[i].scale;
-      d.trunc_k = v[i].trunc_k;
-      d.flags = (v[i].norm == GS_NORM_PEAK ? kFlagPeak : 0) |
-                (v[i].window == GS_WINDOW_RATIO ? kFlagRatio : 0) |
-                (v[i].align == GS_ALIGN_HALF ? kFlagHalf : 0) |
-                (g[i].head ? kFlagHead : 0) |
-                (g[i].head && g[i].head->offset_tanh ? kFlagOffsetTanh : 0);
-      if (g[i].head) {
-        d.h_sigma_lo = g[i].head->sigma_lo;
-        d.h_sigma_span = g[i].head->sigma_span;
-        d.h_rho_scale = g[i].head->rho_scale;
-        d.h_offset_scale = g[i].head->offset_scale;
-      }
-      d.tiles_x = (v[i].out_w + tile - 1) / tile;
-      d.tiles_y = (v[i].out_h + tile - 1) / tile;
       d.t_base = tbase;
       d.p_base = pbase;
       d.b_base = bbase;
@@ -495,13 +503,13 @@ gs_status run_forward(int32_t n_images, const gs_gaussians* g, const gs_view* v,
     // the pairs per tile (into the array the setup kernel cleared) and the
     // reach; the raster sums its tile's count, enumerates the tile's
     // candidates and leaves the tile's list for the adjoint (no sort)
-    e = launch_preprocess(c.w, s);
+    e = launch_preprocess(c.w, describe(g[0], v[0], c.P.tile), s);
     if (e != cudaSuccess) return cuda_fail(e, "preprocess");
     e = launch_raster_fwd(c.w, nullptr, c.P.batch, s);
     if (e != cudaSuccess) return cuda_fail(e, "raster_fwd");
     return GS_OK;
   }
-  e = launch_preprocess(c.w, s);
+  e = launch_preprocess(c.w, describe(g[0], v[0], c.P.tile), s);
   if (e != cudaSuccess) return cuda_fail(e, "preprocess");
   if (c.w.n > 0) {
     e = launch_emit(c.w, s);
@@ -553,7 +561,7 @@ gs_status run_backward(int32_t n_images, const gs_gaussians* g, const gs_view* v
     e = c.w.n_gblocks > 0 ? launch_raster_bwd_gblock(c.w, s) : launch_raster_bwd_gw(c.w, s);
     if (e != cudaSuccess) return cuda_fail(e, "raster_bwd_gw");
   }
-  e = launch_preprocess_bwd(c.w, s);
+  e = launch_preprocess_bwd(c.w, describe(g[0], v[0], c.P.tile), s);
   if (e != cudaSuccess) return cuda_fail(e, "preprocess_bwd");
   return GS_OK;
 }

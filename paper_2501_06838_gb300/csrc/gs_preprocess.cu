@@ -6,6 +6,8 @@
 // Gaussian head (Sec. 3.2) when the arrays hold raw head outputs.
 #include <algorithm>
 
+#include <type_traits>
+
 #include "gs_internal.cuh"
 
 namespace gs {
@@ -17,8 +19,7 @@ constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kLog2TwoPi = 2.6514961294723187f;
 
 __global__ void k_setup(SetupChunk c, Ws w) {
-  griddep_release();
-  griddep_wait();
+  griddep_enter(w);
   const int t = threadIdx.x;
   if (c.reset && w.grid)   // clear the per-tile pair counts of grid binning
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + t; i < w.tiles; i += (int64_t)gridDim.x * blockDim.x)
@@ -79,17 +80,18 @@ struct Phys {
   float D;   // (1 - rho)(1 + rho), formed without cancellation as |rho| -> 1
 };
 
+template <bool L2 = false>
 __device__ __forceinline__ Phys load_gaussian(const ImageDesc& D, int64_t li, float (&raw)[9]) {
   const int dt = D.dtype;
-  raw[0] = load_param(D.off, 2 * li, dt);
-  raw[1] = load_param(D.off, 2 * li + 1, dt);
-  raw[2] = load_param(D.sig, 2 * li, dt);
-  raw[3] = load_param(D.sig, 2 * li + 1, dt);
-  raw[4] = load_param(D.rho, li, dt);
-  raw[5] = load_param(D.rgb, 3 * li, dt);
-  raw[6] = load_param(D.rgb, 3 * li + 1, dt);
-  raw[7] = load_param(D.rgb, 3 * li + 2, dt);
-  raw[8] = load_param(D.alpha, li, dt);
+  raw[0] = load_param<L2>(D.off, 2 * li, dt);
+  raw[1] = load_param<L2>(D.off, 2 * li + 1, dt);
+  raw[2] = load_param<L2>(D.sig, 2 * li, dt);
+  raw[3] = load_param<L2>(D.sig, 2 * li + 1, dt);
+  raw[4] = load_param<L2>(D.rho, li, dt);
+  raw[5] = load_param<L2>(D.rgb, 3 * li, dt);
+  raw[6] = load_param<L2>(D.rgb, 3 * li + 1, dt);
+  raw[7] = load_param<L2>(D.rgb, 3 * li + 2, dt);
+  raw[8] = load_param<L2>(D.alpha, li, dt);
   Phys p;
   if (D.flags & kFlagHead) {
     const bool ot = (D.flags & kFlagOffsetTanh) != 0;
@@ -265,20 +267,31 @@ __device__ __forceinline__ void store_32(float4* p, float4 a, float4 b) {
                : "memory");
 }
 
+// The image descriptors of a pass: the only image's by value (reads_early: the
+// pass reads before its wait), or from the workspace's table.
+struct FromTable {};
+__device__ __forceinline__ const ImageDesc& image_desc(const Ws&, const ImageDesc& one, int) { return one; }
+__device__ __forceinline__ const ImageDesc& image_desc(const Ws& w, FromTable, int im) { return w.images[im]; }
+
 constexpr int kChainBlock = 128;   // Gaussians per chain-rule block
+static_assert(kFootprintBlock == 256, "kOneWave");
 constexpr int kCountBand = 512;   // entries of a warp's tile-count table (grid binning)
 
-__global__ void __launch_bounds__(kFootprintBlock) k_preprocess(Ws w) {
-  griddep_wait();
+template <class One>
+__global__ void __launch_bounds__(kFootprintBlock, 6) k_preprocess(Ws w, const __grid_constant__ One one) {
+  constexpr bool ONE = std::is_same<One, ImageDesc>::value;
+  auto start = [&]() {
+    griddep_wait();
+    // Sorted binning: clear the tile ranges (grid-stride) so empty tiles read
+    // (0, 0). Grid binning: the forward raster writes every tile's range.
+    if (!w.grid)
+      for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < w.tiles;
+           t += (int64_t)gridDim.x * blockDim.x)
+        w.ranges[t] = make_uint2(0u, 0u);
+  };
+  if (!ONE) start();
   __shared__ unsigned long long sw[kFootprintBlock / 32], sp[kFootprintBlock / 32];
   __shared__ int band[kFootprintBlock / 32][kCountBand];   // grid binning: per-warp count table
-  // Sorted binning: clear the tile ranges (grid-stride) so empty tiles read
-  // (0, 0). Grid binning: the forward raster writes every tile's range.
-  if (!w.grid)
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < w.tiles;
-         t += (int64_t)gridDim.x * blockDim.x)
-      w.ranges[t] = make_uint2(0u, 0u);
-
   const int64_t gi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   unsigned long long pix = 0ull;
   uint32_t cnt = 0u;
@@ -287,18 +300,14 @@ __global__ void __launch_bounds__(kFootprintBlock) k_preprocess(Ws w) {
   uint4 trk = make_uint4(0u, 0u, 0u, 0u);  // tile rectangle, for the per-tile counts
   uint32_t tcol0 = 0u;                     // its first tile column in the image
   int tim = -1, tty0 = 0, tty1 = -1;       // its image and tile rows
-  if (gi < w.n) {
-    const int im = image_of_gaussian(w.images, w.n_images, gi);
-    const ImageDesc& D = w.images[im];
+  // the Gaussian's footprint and the record's exponent terms and colour
+  auto compute = [&](const ImageDesc& D, Footprint& F, float4& expo, float4& colour) {
+    const float s = D.scale;
     const int64_t li = gi - D.g_base;
     float raw[9];
-    const Phys P = load_gaussian(D, li, raw);
-    const float sx = P.sx, sy = P.sy, rho = P.rho;
-    const float cr = P.cr, cg = P.cg, cb = P.cb, al = P.al;
-    const float s = D.scale;
-    const Footprint F = footprint(D, li, P);
-    const bool ok = F.ok;
-    const int x0 = F.x0, x1 = F.x1, y0 = F.y0, y1 = F.y1;
+    const Phys P = load_gaussian<ONE>(D, li, raw);
+    const float sx = P.sx, sy = P.sy, rho = P.rho, al = P.al;
+    F = footprint(D, li, P);
     // Records and compact windows stay in image coordinates; tiles are the
     // output's (rows from row0).
 
@@ -317,10 +326,17 @@ __global__ void __launch_bounds__(kFootprintBlock) k_preprocess(Ws w) {
     // Eq. 2 normalisation 1 / (2 pi sx sy sqrt(D)), or 1 for the peak reading.
     const float l = (D.flags & kFlagPeak) == 0 ? -(kLog2TwoPi + log2f(sx) + log2f(sy) + 0.5f * log2f(Dr)) : 0.0f;
 
+    expo = make_float4(sA, sK, gY, l);
+    colour = make_float4(al * P.cr, al * P.cg, al * P.cb, 0.0f);
+  };
+  auto store = [&](const ImageDesc& D, int im, const Footprint& F, float4 expo, float4 colour) {
+    const float s = D.scale;
+    const bool ok = F.ok;
+    const int x0 = F.x0, x1 = F.x1, y0 = F.y0, y1 = F.y1;
     // a record as two 32-byte stores: whole sectors
     float4* rec = w.records + gi * kRecordF4;
-    store_32(rec, make_float4(F.cx_hi, F.cx_lo, F.cy_hi, F.cy_lo), make_float4(sA, sK, gY, l));
-    store_32(rec + 2, make_float4(al * cr, al * cg, al * cb, 0.0f),
+    store_32(rec, make_float4(F.cx_hi, F.cx_lo, F.cy_hi, F.cy_lo), expo);
+    store_32(rec + 2, colour,
              make_float4(__int_as_float(x0), __int_as_float(x1), __int_as_float(y0), __int_as_float(y1)));
 
     if (w.grid) {
@@ -358,6 +374,21 @@ __global__ void __launch_bounds__(kFootprintBlock) k_preprocess(Ws w) {
     }
     trk = tr;
     if (!ok) atomicOr(&w.hdr->status, kStInvalid);
+  };
+  {
+    Footprint F;
+    float4 expo, colour;
+    if (ONE) {
+      const ImageDesc& D = image_desc(w, one, 0);
+      if (gi < w.n) compute(D, F, expo, colour);
+      start();
+      if (gi < w.n) store(D, 0, F, expo, colour);
+    } else if (gi < w.n) {
+      const int im = image_of_gaussian(w.images, w.n_images, gi);
+      const ImageDesc& D = image_desc(w, one, im);
+      compute(D, F, expo, colour);
+      store(D, im, F, expo, colour);
+    }
   }
   if (w.grid) {
     // pairs per tile, as per-row differences: +1 at the rectangle's first
@@ -395,7 +426,7 @@ __global__ void __launch_bounds__(kFootprintBlock) k_preprocess(Ws w) {
         }
       }
       __syncwarp();
-      const int64_t base = w.images[imL].t_base + (int64_t)RY0 * tilesx + CX0;
+      const int64_t base = (ONE ? 0 : w.images[imL].t_base) + (int64_t)RY0 * tilesx + CX0;
       for (int e = lane; e < span; e += 32) {
         const int v = h[e];
         if (v != 0) {
@@ -518,22 +549,42 @@ __global__ void __launch_bounds__(kFootprintBlock) k_count(Ws w) {
 // dsK/drho = r / (s sy D), dl/drho = rho / (D ln2)), and cx = s mu_x.
 // No term cancels at order 1/D^2 as |rho| -> 1, which the same chain rule in
 // the moments of X would.
-// The gradients of Gaussian gi (0 where its window is empty).
-__device__ __forceinline__ void chain_rule(const Ws& w, int64_t gi, float (&gr)[9]) {
-  const int im = image_of_gaussian(w.images, w.n_images, gi);
-  const ImageDesc& D = w.images[im];
+// The gradients of Gaussian gi of image D (0 where its window is empty). ONE:
+// everything but the moments is read before the wait for the adjoint.
+template <bool ONE>
+__device__ __forceinline__ void chain_rule(const Ws& w, const ImageDesc& D, int64_t gi, float (&gr)[9]) {
   const int64_t li = gi - D.g_base;
 #pragma unroll
   for (int k = 0; k < 9; ++k) gr[k] = 0.0f;
-  const float4* rec = w.records + gi * kRecordF4;
-  // every load that does not depend on the image table, issued together
-  const float4* gm = reinterpret_cast<const float4*>(w.grec + gi * 12);
-  const float4 r3 = rec[3], rc = rec[2], m0 = gm[0], m1 = gm[1];
-  const bool live = __float_as_int(r3.x) <= __float_as_int(r3.y) &&
-                    __float_as_int(r3.z) <= __float_as_int(r3.w);
-  if (!live) return;
+  const bool in = gi < w.n;
+  const float4* rec = w.records + (in ? gi : 0) * kRecordF4;
+  const float4* gm = reinterpret_cast<const float4*>(w.grec + (in ? gi : 0) * 12);
+  float4 r3, rc, m0, m1;
   float raw[9];
-  const Phys P = load_gaussian(D, li, raw);
+  Phys P;
+  bool live = false;
+  if (in) {
+    // every load that does not depend on the image table, issued together
+    if (ONE) {
+      r3 = __ldcg(rec + 3);
+      rc = __ldcg(rec + 2);
+      P = load_gaussian<true>(D, li, raw);
+    } else {
+      r3 = rec[3];
+      rc = rec[2];
+      m0 = gm[0];
+      m1 = gm[1];
+    }
+    live = __float_as_int(r3.x) <= __float_as_int(r3.y) && __float_as_int(r3.z) <= __float_as_int(r3.w);
+  }
+  if (ONE) griddep_wait();
+  if (!live) return;
+  if (ONE) {
+    m0 = gm[0];
+    m1 = gm[1];
+  } else {
+    P = load_gaussian(D, li, raw);
+  }
   const float sx = P.sx, sy = P.sy, rho = P.rho;
   const float cr = P.cr, cg = P.cg, cb = P.cb, al = P.al;
   const float s = D.scale;
@@ -571,27 +622,28 @@ __device__ __forceinline__ void chain_rule(const Ws& w, int64_t gi, float (&gr)[
 // Gaussian instead of 2.6, and the stores bounded the kernel: 32.7 -> 22.4 us on
 // 518,400 Gaussians (60 MB in and out: 2.7 TB/s), 18.3 -> 12.0 on 220,052 and
 // 10.3 -> 7.9 on 65,536, where the loads' latency is what is left.
-__global__ void __launch_bounds__(kChainBlock) k_preprocess_bwd(Ws w) {
+template <class One>
+__global__ void __launch_bounds__(kChainBlock) k_preprocess_bwd(Ws w, const __grid_constant__ One one) {
+  constexpr bool ONE = std::is_same<One, ImageDesc>::value;
   griddep_release();
-  griddep_wait();
+  if (!ONE) griddep_wait();
   __shared__ float sg[kChainBlock * 9];
   const int64_t g0 = blockIdx.x * (int64_t)kChainBlock, gi = g0 + threadIdx.x;
-  if (gi == 0) w.hdr->bwd_counter = 0u;   // the next adjoint of this forward starts at tile 0
   const int rows = (int)min((int64_t)kChainBlock, w.n - g0);
-  if (gi < w.n) {
+  {
     float gr[9];
-    chain_rule(w, gi, gr);
+    chain_rule<ONE>(w, image_desc(w, one, ONE ? 0 : image_of_gaussian(w.images, w.n_images, gi)), gi, gr);
 #pragma unroll
     for (int k = 0; k < 9; ++k) sg[threadIdx.x * 9 + k] = gr[k];
   }
+  if (gi == 0) w.hdr->bwd_counter = 0u;   // the next adjoint of this forward starts at tile 0
   __syncthreads();   // every accumulator row of the block has been read
   // cleared for the next adjoint of the same forward (the tile adjoint adds)
   float4* z = reinterpret_cast<float4*>(w.grec + g0 * 12);
   for (int i = threadIdx.x; i < 3 * rows; i += kChainBlock) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   // the block's images one after the other (mostly one)
   for (int r0 = 0; r0 < rows;) {
-    const int im = image_of_gaussian(w.images, w.n_images, g0 + r0);
-    const ImageDesc& D = w.images[im];
+    const ImageDesc& D = image_desc(w, one, ONE ? 0 : image_of_gaussian(w.images, w.n_images, g0 + r0));
     const int r1 = (int)min((int64_t)rows, D.g_base + D.n - g0);
     float* out = (w.direct ? w.grads0 : D.grads) + (g0 + r0 - D.g_base) * 9;
     for (int i = threadIdx.x; i < 9 * (r1 - r0); i += kChainBlock) out[i] = sg[9 * r0 + i];
@@ -608,12 +660,14 @@ cudaError_t launch_setup(const SetupChunk& c, const Ws& w, cudaStream_t s) {
   return launch_chain(k_setup, dim3(blocks), dim3(256), 0, s, c, w);
 }
 
-cudaError_t launch_preprocess(const Ws& w, cudaStream_t s) {
+cudaError_t launch_preprocess(const Ws& w, const ImageDesc& first, cudaStream_t s) {
   int64_t work = w.n > (int64_t)w.tiles ? w.n : (int64_t)w.tiles;
   int blocks = (int)((work + kFootprintBlock - 1) / kFootprintBlock);
   if (blocks < 1) blocks = 1;
   LaunchScope ls(kKPreprocess, s);
-  return launch_chain(k_preprocess, dim3(blocks), dim3(kFootprintBlock), 0, s, w);
+  if (reads_early(w))
+    return launch_chain(k_preprocess<ImageDesc>, dim3(blocks), dim3(kFootprintBlock), 0, s, w, first);
+  return launch_chain(k_preprocess<FromTable>, dim3(blocks), dim3(kFootprintBlock), 0, s, w, FromTable());
 }
 
 cudaError_t launch_count(const Ws& w, cudaStream_t s) {
@@ -623,11 +677,13 @@ cudaError_t launch_count(const Ws& w, cudaStream_t s) {
   return launch_chain(k_count, dim3((unsigned)blocks), dim3(kFootprintBlock), 0, s, w);
 }
 
-cudaError_t launch_preprocess_bwd(const Ws& w, cudaStream_t s) {
+cudaError_t launch_preprocess_bwd(const Ws& w, const ImageDesc& first, cudaStream_t s) {
   if (w.n == 0) return cudaSuccess;
   const int blocks = (int)((w.n + kChainBlock - 1) / kChainBlock);
   LaunchScope ls(kKPreprocessBwd, s);
-  return launch_chain(k_preprocess_bwd, dim3(blocks), dim3(kChainBlock), 0, s, w);
+  if (reads_early(w))
+    return launch_chain(k_preprocess_bwd<ImageDesc>, dim3(blocks), dim3(kChainBlock), 0, s, w, first);
+  return launch_chain(k_preprocess_bwd<FromTable>, dim3(blocks), dim3(kChainBlock), 0, s, w, FromTable());
 }
 
 }  // namespace gs
