@@ -5,7 +5,6 @@
 // Both read the parameters through load_gaussian, which applies the fused
 // Gaussian head (Sec. 3.2) when the arrays hold raw head outputs.
 #include <algorithm>
-
 #include <type_traits>
 
 #include "gs_internal.cuh"
