@@ -59,15 +59,15 @@ PAIR_CYCLES = {"raster_fwd": 6.5, "raster_bwd": 12.0, "raster_bwd_gw": 12.0}
 # source they were taken on: reported as null once that source file changes.
 TRAFFIC = {
     ("c2", "raster_bwd"): ("gs_adjoint_tile.cu",
-                           "d329f4b6381f0a3278e01aa6c5f2dc462ed321c7207134b08b7a6235270e4c31",
-                           21309184 + 0, "profiles/raster_bwd_c2_1024x1024.md"),
+                           "73b41edd332ba9febab557472d55993aae9f872c51f833f52eabf6470f7129c8",
+                           21310464 + 0, "profiles/raster_bwd_c2_1024x1024.md"),
     ("c4x12-bf16", "raster_bwd"): ("gs_adjoint_tile.cu",
-                                   "d329f4b6381f0a3278e01aa6c5f2dc462ed321c7207134b08b7a6235270e4c31",
-                                   349436928 + 20665088,
+                                   "73b41edd332ba9febab557472d55993aae9f872c51f833f52eabf6470f7129c8",
+                                   350463232 + 21343232,
                                    "profiles/raster_bwd_c4x12_bf16_5760x3240.md"),
     ("c4x12-bf16", "raster_fwd"): ("gs_raster.cu",
-                                   "a1d3fc604d7d88dbb6ddcab89fd2d676a52d2fe9dd3e9fb2e164cfe5074db27f",
-                                   37752320 + 233056512,
+                                   "a95c3034d515891c5963cdcecba72fa137b9f1305d03a3e65ba853faa2938bbc",
+                                   37670656 + 227392256,
                                    "profiles/raster_fwd_c4x12_bf16_5760x3240.md"),
 }
 

@@ -3,8 +3,9 @@
 // adjoint, one lane per Gaussian over a tile's pixels, is gs_adjoint_tile.cu.)
 //
 // Tile 16, one warp per tile: k_raster_fwd16 (the tile in four strips, below);
-// one warp per pair of tiles: k_raster_fwd_pair. The rest of this comment is
-// the layout of tiles 8 and 32, k_raster_fwd:
+// one warp per pair of tiles: k_raster_fwd_pair; several warps per tile:
+// k_raster_fwd_team. The rest of this comment is the layout of tiles 8 and 32,
+// k_raster_fwd:
 // one CTA of NT = TILE*TILE/BY threads renders one TILE x TILE tile of HR
 // pixels; thread t owns column t % TILE and the BY consecutive rows
 // [(t / TILE) * BY, + BY). The tile's Gaussians (a contiguous run of the sorted
@@ -334,7 +335,10 @@ __device__ __forceinline__ void fwd_gaussian(float2 (&acc)[NQ][3], const FwdOps<
 // against it: 41.2 -> 34.4 us on 65,536 Gaussians at 1024 x 1024 (windows of
 // 22 px on average: 0.68 of the tile's columns per Gaussian), 81.8 -> 53.5 us
 // on 220,052 at 1002 x 751 (14 px), 4134 -> 3776 us on 518,400 at 720 x 720
-// under the ratio window (144 px).
+// under the ratio window (144 px). Ids run along LR rows, so a batch's windows
+// share rows and spread over the columns: strips of whole columns are evenly
+// filled. Strips cut in halves of 8 rows (51 us at 1002 x 751 against 50) or
+// tiles cut in quadrants (54) were not.
 // ---------------------------------------------------------------------------
 constexpr int kStripSlots = 33;   // 32 slots and, in front, one that adds nothing (odd: no bank conflicts)
 
