@@ -291,7 +291,8 @@ int radix_passes(int64_t tiles) { return (key_bits(tiles) + 8) / 9; }
 // together pays already. Measured, one warp -> team: ratio window, 2,025 tiles
 // with lists of 23,000 3.73 -> 2.99 ms (8 warps: 3.11), 8,100 tiles with 6,400
 // 3.08 -> 2.94 ms, 2,025 tiles with 1,500 320 -> 263 us, 250 tiles with 4,000 to
-// 10,000 547 -> 117 us (4 warps: 154); boxes, us, at 100 to 729 tiles: 96
+// 10,000 547 -> 108 us (4 warps: 154); boxes, us, at 100 to 729 tiles (teams of 8
+// with the registers of 4; they are 7% to 11% faster now): 96
 // Gaussians per tile 86.8 -> 40.6, 64 77.8 -> 48.7, 24 34.9 -> 28.9, 16 no change;
 // at 3,249 tiles: 643 516 -> 431, 251 331 -> 306, 140 183 -> 211; at 15,625 tiles:
 // 655 2000 -> 1973, 455 1014 -> 1127.

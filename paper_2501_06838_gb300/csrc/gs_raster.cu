@@ -751,7 +751,7 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
 // What bounds it: the strips' arithmetic, once enough warps run. One warp per
 // tile left 2,025 tiles with lists of 23,000 at 3 or 4 warps per scheduler (the
 // fuller ones last: 3.73 ms; teams of four: 2.99) and 250 tiles with lists of
-// 4,000 to 10,000 waiting for the longest (514 us; teams of eight: 117). The
+// 4,000 to 10,000 waiting for the longest (514 us; teams of eight: 108). The
 // host's rule says where a team runs and what else was measured.
 // ---------------------------------------------------------------------------
 struct TeamWarp {
@@ -774,8 +774,13 @@ struct ListSource {
   }
 };
 
+// Two CTAs of eight per SM are all that fit: with the 128 registers that this
+// leaves instead of 86, 250 tiles with lists of 4,000 to 10,000 take 108 instead
+// of 116 us and 64 to 225 tiles of k-sigma boxes 7% to 11% less. For four warps
+// the compiler's own choice (96) is the best: 2.90 ms on the paper's 2,025
+// tiles, 2.99 with five CTAs asked for, 3.10 with one.
 template <int NW, bool GRID>
-__global__ void __launch_bounds__(NW * 32) k_raster_fwd_team(Ws w, const uint32_t* vals) {
+__global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 0) k_raster_fwd_team(Ws w, const uint32_t* vals) {
   griddep_release();
   griddep_wait();
   constexpr int NT = NW * 32, PER = 768 / NT;
