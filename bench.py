@@ -60,14 +60,14 @@ PAIR_CYCLES = {"raster_fwd": 6.5, "raster_bwd": 12.0, "raster_bwd_gw": 12.0}
 TRAFFIC = {
     ("c2", "raster_bwd"): ("gs_adjoint_tile.cu",
                            "73b41edd332ba9febab557472d55993aae9f872c51f833f52eabf6470f7129c8",
-                           21310464 + 0, "profiles/raster_bwd_c2_1024x1024.md"),
+                           21310976 + 0, "profiles/raster_bwd_c2_1024x1024.md"),
     ("c4x12-bf16", "raster_bwd"): ("gs_adjoint_tile.cu",
                                    "73b41edd332ba9febab557472d55993aae9f872c51f833f52eabf6470f7129c8",
-                                   350463232 + 21343232,
+                                   350088704 + 21108480,
                                    "profiles/raster_bwd_c4x12_bf16_5760x3240.md"),
     ("c4x12-bf16", "raster_fwd"): ("gs_raster.cu",
-                                   "a95c3034d515891c5963cdcecba72fa137b9f1305d03a3e65ba853faa2938bbc",
-                                   37670656 + 227392256,
+                                   "7d54d7101ecc6906751ede1a417846269f59e94b1bca9ef0d6d2255aa3bf690d",
+                                   37683968 + 227410432,
                                    "profiles/raster_fwd_c4x12_bf16_5760x3240.md"),
 }
 
