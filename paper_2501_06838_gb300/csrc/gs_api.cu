@@ -124,6 +124,7 @@ struct Problem {
   int64_t n;
   int64_t tiles;
   int64_t tile_pairs;   // horizontal pairs of tiles
+  double listed;        // expected list entries of all tiles (k-sigma boxes; see validate)
   int tile, batch;
   int adjoint;   // gs_adjoint resolved: 1 tile, 2 Gaussian-warp, 3 tile quadrants
   int grid;      // gs_binning resolved: 1 grid-implicit, 0 sorted pair list
@@ -139,11 +140,15 @@ struct Problem {
 // 84.2; 4 per pixel (sigma up to 3) at scale 8, 2,850 pairs 125 / 138, 6,441 255
 // / 244, at scale 4, 13,366 pairs 690 / 727; 16 per pixel at scale 8, 6,441 pairs
 // 677 / 730. Below 256 pairs either layout is one short round of warps on part of
-// the chip (tiles 12 to 14 us, pairs 13 to 16): the large scales keep pairs.
-bool pairs_pay(int64_t pairs, int64_t n, int64_t tiles, float scale) {
+// the chip, and tiles (with teams where lists are longer) are faster: one image,
+// calls, 4 Gaussians per pixel at scale 12 19.3 / 26.4, 1 per pixel at scale 6
+// 12.7 / 14.6. Only batches of small images with short lists keep the pairs that
+// a scale of 6 always had (4 images, 10.3 to 15.9 / 12.1 to 20.0).
+bool pairs_pay(const Problem& P, float scale) {
+  const int64_t pairs = P.tile_pairs, n = P.n, tiles = P.tiles;
   if (scale >= 4.0f && pairs >= 5000) return n < (scale >= 6.0f ? 30 : 18) * tiles;
   if (scale >= 10.0f && pairs >= 1200) return n < 8 * tiles;
-  return scale >= 6.0f && pairs < 256 && n < 8 * tiles;
+  return scale >= 6.0f && pairs < 256 && P.n_images > 1 && P.listed < 60.0 * tiles;
 }
 
 gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Problem* P) {
@@ -153,6 +158,7 @@ gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Pr
   P->n = 0;
   P->tiles = 0;
   P->tile_pairs = 0;
+  P->listed = 0.0;
   P->tile = tile_of(v[0]);
   P->batch = batch_of(v[0]);
   bool grid_ok = true;   // every image on a reference grid, coordinates fit int16
@@ -216,6 +222,10 @@ gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Pr
     P->n += G.n;
     P->tiles += tx * ty;
     P->tile_pairs += (tx + 1) / 2 * ty;
+    // a tile takes the Gaussians of its own LR pixels and, with sigma about 0.8 LR
+    // pixels at 3 sigma, of 2.4 more on each side
+    const double per = 1.0 + 0.3 * (double)V.scale;
+    P->listed += (double)G.n * per * per;
   }
   if (!(P->tile == 8 || P->tile == 16 || P->tile == 32))
     return fail(GS_ERR_INVALID, "tile must be 8, 16 or 32 (got %lld)", (long long)P->tile);
@@ -238,7 +248,7 @@ gs_status validate(int32_t n_images, const gs_gaussians* g, const gs_view* v, Pr
     return fail(GS_ERR_UNSUPPORTED, "raster PAIR needs grid binning and tile 16");
   P->pair = (v[0].raster == GS_RASTER_PAIR ||
              (v[0].raster == GS_RASTER_AUTO && pair_ok && sigma_windows &&
-              pairs_pay(P->tile_pairs, P->n, P->tiles, max_scale))) ? 1 : 0;
+              pairs_pay(*P, max_scale))) ? 1 : 0;
   if (v[0].adjoint == GS_ADJOINT_QUADRANT && P->tile != 16)
     return fail(GS_ERR_UNSUPPORTED, "adjoint QUADRANT needs tile 16");
   // AUTO: quadrants at tile 16 where every view has truncated SIGMA windows and
@@ -288,14 +298,19 @@ int radix_passes(int64_t tiles) { return (key_bits(tiles) + 8) / 9; }
 // bounded below by the Gaussians per tile (lists are 3 to 9 times that). Where
 // the tiles are few enough for all teams to be resident at once (2 of 8 warps or
 // 5 of 4 per SM, 152 SMs) idle warps take nobody's place, and building the list
-// together pays already. Measured, one warp -> team: ratio window, 2,025 tiles
-// with lists of 23,000 3.73 -> 2.99 ms (8 warps: 3.11), 8,100 tiles with 6,400
-// 3.08 -> 2.94 ms, 2,025 tiles with 1,500 320 -> 263 us, 250 tiles with 4,000 to
-// 10,000 547 -> 108 us (4 warps: 154); boxes, us, at 100 to 729 tiles (teams of 8
-// with the registers of 4; they are 7% to 11% faster now): 96
-// Gaussians per tile 86.8 -> 40.6, 64 77.8 -> 48.7, 24 34.9 -> 28.9, 16 no change;
-// at 3,249 tiles: 643 516 -> 431, 251 331 -> 306, 140 183 -> 211; at 15,625 tiles:
-// 655 2000 -> 1973, 455 1014 -> 1127.
+// together pays already: from 20 Gaussians per tile, or where the lists that
+// their scale leads one to expect are long enough (Problem::listed). Measured,
+// one warp -> team. Ratio window: 2,025 tiles with lists of 23,000 3.73 -> 2.90
+// ms (8 warps: 3.11), 8,100 tiles with 6,400 3.08 -> 2.94 ms, 2,025 tiles with
+// 1,500 320 -> 263 us, 250 tiles with 4,000 to 10,000 547 -> 108 us (4 warps:
+// 154). Boxes, forward, us, on 100 to 729 tiles by Gaussians per tile (teams of 8
+// with the registers of 4; they are 7% to 11% faster now): 96 86.8 -> 40.6, 64
+// 77.8 -> 48.7, 24 34.9 -> 28.9. Boxes, calls, on up to 304 tiles by expected
+// list: 150 22.7 -> 19.3, 120 20.5 -> 18.7, 77 14.7 -> 14.1, 64 14.2 -> 13.9, 50 to
+// 56 13.5 -> 13.6, 37 12.1 -> 12.5; on 400 to 702 tiles (4 warps): 185 26.4 ->
+// 25.4, 77 15.7 -> 16.0, 56 15.3 -> 17.0. Boxes on 3,249 tiles by Gaussians per
+// tile: 643 516 -> 431, 251 331 -> 306, 140 183 -> 211; on 15,625: 655 2000 ->
+// 1973, 455 1014 -> 1127.
 int team_of(const Problem& P, const gs_gaussians* g, const gs_view* v) {
   if (P.tile != 16 || P.pair || P.batch == 64) return 0;
   double listed = 0.0;
@@ -317,7 +332,8 @@ int team_of(const Problem& P, const gs_gaussians* g, const gs_view* v) {
   listed /= (double)P.tiles;
   const bool few = P.tiles <= 760;
   const double line = known ? (few ? 512.0 : 1024.0) : few ? 20.0 : P.tiles <= 3300 ? 240.0 : 600.0;
-  if (listed < line) return 0;
+  const bool lists = !known && few && P.listed >= (P.tiles <= 304 ? 60.0 : 150.0) * (double)P.tiles;
+  if (listed < line && !lists) return 0;
   return P.tiles <= 304 ? 8 : 4;
 }
 

@@ -24,6 +24,8 @@ CASES = {
     "ratio_many_tiles": (48, 52, 9, dict(scale=9.3, trunc_k=0.25, window=S.WINDOW_RATIO)),
     "dense_sigma": (30, 34, 16, dict(scale=1.3)),
     "sparse_sigma": (20, 24, 4, dict(scale=4.6)),        # 45 Gaussians per tile: lists below a segment
+    "thin_sigma": (24, 24, 1, dict(scale=4.0)),          # 16 per tile, lists of about 75
+    "wide_sigma": (11, 14, 4, dict(scale=12.0)),         # 6 per tile, lists of about 130
     "many_tiles_sigma": (112, 113, 9, dict(scale=4.0)),  # 783 tiles, 145 per tile: one warp
     "many_tiles_team": (150, 151, 9, dict(scale=3.0)),   # 841 tiles, 242 per tile: teams again
 }
