@@ -130,7 +130,8 @@ typedef enum {
  *         that reach and tests their windows. No sort: the forward leaves each
  *         tile's list in the workspace for the adjoint (one 4-byte array of
  *         pair capacity instead of four). Needs ref_grid_m > 0 for every image
- *         and outputs of at most 32767 px a side (GS_ERR_UNSUPPORTED otherwise);
+ *         and outputs of at most 32767 px a side, bands of any rows among them
+ *         (GS_ERR_UNSUPPORTED otherwise);
  *   AUTO: GRID where it applies, else SORT.
  * Both give every tile the same Gaussians in the same (ascending id) order, so
  * the forward is bitwise the same. */

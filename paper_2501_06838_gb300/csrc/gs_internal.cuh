@@ -94,7 +94,8 @@ struct Ws {
   uint32_t* hscan;            // [radix] per-digit totals
   uint2* ranges;              // [T]
   float* grec;                // [N][12] record-space gradient moments
-  short4* win;                // [N] windows (x0, y0, x1, y1) for grid binning (empty: never meets a tile)
+  short4* win;                // [N] windows (x0, y0, x1, y1) for grid binning, in output rows (from
+                              // row0; empty: never meets a tile)
   int4* ext;                  // [n_images] reach (DL, DR, DT, DB) of the windows past their LR cell, HR px
   uint32_t* tcount;           // [T] grid mode: per-row differences of the (tile, Gaussian)
                               // pairs per tile (a tile's count is the prefix along its row)

@@ -307,8 +307,8 @@ __global__ void __launch_bounds__(kFootprintBlock, 6) k_preprocess(Ws w, const _
     const Phys P = load_gaussian<ONE>(D, li, raw);
     const float sx = P.sx, sy = P.sy, rho = P.rho, al = P.al;
     F = footprint(D, li, P);
-    // Records and compact windows stay in image coordinates; tiles are the
-    // output's (rows from row0).
+    // Records stay in image coordinates; tiles and the compact windows are the
+    // output's (rows from row0: 16 bits hold a band wherever it lies).
 
     // Exponent in HR pixels and log2 units: -q/2 of Eq. 2 times log2(e), with
     // u = X/s, v = Y/s, written with the square completed in X so that no
@@ -342,15 +342,17 @@ __global__ void __launch_bounds__(kFootprintBlock, 6) k_preprocess(Ws w, const _
       // compact window for the tile test, and how far it reaches past the
       // Gaussian's LR cell (i, j): DL = s j - x0, DR = x1 - s j (rows alike),
       // rounded up, plus one pixel of margin for the float32 rounding of s j
+      // (more rows where a band lies so far down that they round to more)
       const bool live = x0 <= x1 && y0 <= y1;
-      w.win[gi] = live ? make_short4((short)x0, (short)y0, (short)x1, (short)y1)
+      w.win[gi] = live ? make_short4((short)x0, (short)(y0 - D.row0), (short)x1, (short)(y1 - D.row0))
                        : make_short4(32767, 32767, -32768, -32768);
       if (live) {
         const float sj = s * (float)F.j, si = s * (float)F.i;
         reach.x = max(0, (int)ceilf(sj - (float)x0) + 1);
         reach.y = max(0, (int)ceilf((float)x1 - sj) + 1);
-        reach.z = max(0, (int)ceilf(si - (float)y0) + 1);
-        reach.w = max(0, (int)ceilf((float)y1 - si) + 1);
+        const int margin = 1 + (D.row0 >> 20);
+        reach.z = max(0, (int)ceilf(si - (float)y0) + margin);
+        reach.w = max(0, (int)ceilf((float)y1 - si) + margin);
         rim = im;
       }
     }

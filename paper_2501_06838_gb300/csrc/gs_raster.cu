@@ -129,7 +129,7 @@ struct Candidates {
   int L, total, cur;     // candidates per row, in all, next to test
   uint32_t gid, wrap;    // this lane's candidate; from a row's end to the next row's start
   int col;               // its position in its row
-  uint32_t lo, hi;       // the region: (X0, Y0) and (X1, Y1)
+  uint32_t lo, hi;       // the region: (X0, Y0) and (X1, Y1), output rows
   // to candidate `from` (lane 0's)
   __device__ __forceinline__ void seek(int from) {
     const int c = from + (int)(threadIdx.x & 31);
@@ -214,7 +214,8 @@ struct GridSource {
 // GridSource). A Gaussian of column j meets it only if s j - DL < x0 <= X1 and
 // s j + DR > x1 >= X0; the reach (DL, DR, DT, DB) carries a pixel of margin,
 // far more than the float32 rounding of these quotients, so floor/ceil bound
-// the cells exactly.
+// the cells exactly. Y0 and Y1 are image rows; the windows and the region they
+// are tested against are output rows (from row0), which fit 16 bits.
 __device__ __forceinline__ void candidate_box(const Ws& w, const ImageDesc* D, int X0, int X1,
                                               int Y0, int Y1, Candidates& c) {
   const int4 e = w.ext[D - w.images];   // HR px
@@ -228,7 +229,7 @@ __device__ __forceinline__ void candidate_box(const Ws& w, const ImageDesc* D, i
   c.rb0 = D->g_base + ((int64_t)i0 * D->lr_w + j0) * D->m;
   c.L = (j1 - j0 + 1) * D->m;
   c.total = (j0 <= j1 && i0 <= i1) ? (i1 - i0 + 1) * c.L : 0;
-  c.start(X0, X1, Y0, Y1);
+  c.start(X0, X1, Y0 - D->row0, Y1 - D->row0);
 }
 
 template <int TILE, int NT, int PF>
