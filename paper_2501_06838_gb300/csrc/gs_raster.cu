@@ -638,7 +638,6 @@ template <int PF, bool GRID>
 __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals) {
   griddep_release();
   griddep_wait();
-  constexpr int BATCH = 32 * PF;
   __shared__ __align__(16) float4 raw[PF][4 * 32];
   __shared__ StripTables<1> T[PF];
   __shared__ uint32_t qbuf[GRID ? GridSource<32, PF>::QCAP : 1];
@@ -660,7 +659,7 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
   typename std::conditional<GRID, GridSource<32, PF>, SortedSource<32, PF>>::type src;
   // grid mode: the tile's slice [lbase, lbase + lcount) of the pair list, where
   // the forward leaves its Gaussian ids (ascending) for the adjoint
-  int lbase = 0, lcount = 0, lpos = 0;
+  int lbase = 0, lcount = 0;
   bool lok = false;
   if constexpr (GRID) {
     grid_source_init<16, 32, PF>(w, D, ox, oy, qbuf, src);
@@ -689,10 +688,16 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
     src.pos = (int)range.x;
     src.end = (int)range.y;
   }
-  // grid mode: append a batch of ids to the tile's slice of the list
-  auto keep = [&](const uint32_t (&ids)[PF], int n) {
+  int total;   // the tile's Gaussians (grid mode: the footprint count)
+  if constexpr (GRID) total = lcount; else total = src.end - src.pos;
+  // the next batch's ids, appended in grid mode to the tile's slice of the list
+  int got = 0;
+  uint32_t gid[PF];
+  auto take = [&]() -> int {
+    if (got >= total) return 0;
+    const int n = src.next(gid);
     if constexpr (GRID) {
-      if (lpos + n > lcount) {   // the footprint count and the tile test disagree
+      if (got + n > lcount) {   // the footprint count and the tile test disagree
         if (lane == 0) atomicOr(&w.hdr->status, kStInternal);
         lok = false;
       }
@@ -700,26 +705,22 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
 #pragma unroll
         for (int j = 0; j < PF; ++j) {
           const int i = j * 32 + lane;
-          if (i < n) w.vals[0][lbase + lpos + i] = ids[j];
+          if (i < n) w.vals[0][lbase + got + i] = gid[j];
         }
       }
-      lpos += n;
     }
+    got += n;
+    return n;
   };
-  // batches of the tile's `total` Gaussians (grid mode: the footprint count)
-  int total;
-  if constexpr (GRID) total = lcount; else total = src.end - src.pos;
-  const int nbat = (total + BATCH - 1) / BATCH;
-  uint32_t gid[PF];
-  if (nbat > 0) {
-    keep(gid, src.next(gid));                              // batch 0
-    issue_slots<PF>(w, gid, min(BATCH, total), raw);
-    if (nbat > 1) keep(gid, src.next(gid));                // batch 1
+  int nb = take(), nn = 0;   // entries of this batch and of the next
+  if (nb > 0) {
+    issue_slots<PF>(w, gid, nb, raw);
+    nn = take();
   }
-  for (int b = 0; b < nbat; ++b) {
-    const int nb = min(BATCH, total - b * BATCH);
-    if (b > 0 && b % (kSeg / BATCH) == 0)
-      fold_strips<1>(D, acc, T[0], ox, oy - D->row0, true, b > kSeg / BATCH);   // a segment ends
+  int done = 0;   // entries summed
+  while (nb > 0) {
+    if (done > 0 && done % kSeg == 0)
+      fold_strips<1>(D, acc, T[0], ox, oy - D->row0, true, done > kSeg);   // a segment ends
     cp_async_wait_all();
     __syncwarp();
     StripMasks ms[PF];
@@ -727,16 +728,23 @@ __global__ void __launch_bounds__(32) k_raster_fwd16(Ws w, const uint32_t* vals)
     for (int j = 0; j < PF; ++j)
       ms[j] = strip_masks(stage_strips<1>(raw[j], lane, j * 32 + 31 - lane < nb, ox, oy, T[j]), strip);
     __syncwarp();
-    if (b + 1 < nbat) {
-      issue_slots<PF>(w, gid, min(BATCH, total - (b + 1) * BATCH), raw);
-      if (b + 2 < nbat) keep(gid, src.next(gid));          // batch b + 2
+    int n2 = 0;
+    if (nn > 0) {
+      issue_slots<PF>(w, gid, nn, raw);
+      n2 = take();
     }
 #pragma unroll
     for (int j = 0; j < PF; ++j) walk_strips<1>(acc, ms[j], strip, rp, T[j]);
     __syncwarp();
+    done += nb;
+    nb = nn;
+    nn = n2;
+  }
+  if constexpr (GRID) {   // fewer found than counted: the list is incomplete
+    if (got < total && lane == 0) atomicOr(&w.hdr->status, kStInternal);
   }
 
-  if (total > kSeg)
+  if (done > kSeg)
     fold_strips<1>(D, acc, T[0], ox, oy - D->row0, true, true);
   else
     store_strips<1>(D, acc, T[0], ox, oy - D->row0);
@@ -973,7 +981,7 @@ __global__ void __launch_bounds__(TILE * TILE / BY) k_raster_fwd(Ws w, const uin
   // grid mode: the tile's slice [lbase, lbase + lcount) of the pair list, where
   // the forward leaves its Gaussian ids (ascending) for the adjoint
   __shared__ int sl_base;
-  int lbase = 0, lcount = 0, lpos = 0;
+  int lbase = 0, lcount = 0;
   bool lok = false;
   if constexpr (GRID) {
     grid_source_init<TILE, NT, PF>(w, D, ox, oy, qbuf, src);
@@ -1004,10 +1012,16 @@ __global__ void __launch_bounds__(TILE * TILE / BY) k_raster_fwd(Ws w, const uin
     src.pos = (int)range.x;
     src.end = (int)range.y;
   }
-  // grid mode: append a batch of ids to the tile's slice of the list
-  auto keep = [&](const uint32_t (&ids)[PF], int n) {
+  int total;   // the tile's Gaussians (grid mode: the footprint count)
+  if constexpr (GRID) total = lcount; else total = src.end - src.pos;
+  // the next batch's ids, appended in grid mode to the tile's slice of the list
+  int got = 0;
+  uint32_t gid[PF];
+  auto take = [&]() -> int {
+    if (got >= total) return 0;
+    const int n = src.next(gid);
     if constexpr (GRID) {
-      if (lpos + n > lcount) {   // the footprint count and the tile test disagree
+      if (got + n > lcount) {   // the footprint count and the tile test disagree
         if (threadIdx.x == 0) atomicOr(&w.hdr->status, kStInternal);
         lok = false;
       }
@@ -1015,33 +1029,29 @@ __global__ void __launch_bounds__(TILE * TILE / BY) k_raster_fwd(Ws w, const uin
 #pragma unroll
         for (int j = 0; j < PF; ++j) {
           const int i = j * NT + threadIdx.x;
-          if (i < n) w.vals[0][lbase + lpos + i] = ids[j];
+          if (i < n) w.vals[0][lbase + got + i] = gid[j];
         }
       }
-      lpos += n;
     }
+    got += n;
+    return n;
   };
-  // batches of the tile's `total` Gaussians (grid mode: the footprint count)
-  int total;
-  if constexpr (GRID) total = lcount; else total = src.end - src.pos;
-  const int nbat = (total + BATCH - 1) / BATCH;
-  uint32_t gid[PF];
-  if (nbat > 0) {
-    keep(gid, src.next(gid));                              // batch 0
-    issue_records<NT, PF>(w, gid, min(BATCH, total), raw[0]);
-    if (nbat > 1) keep(gid, src.next(gid));                // batch 1
+  int nb = take(), nn = 0;   // entries of this batch and of the next
+  if (nb > 0) {
+    issue_records<NT, PF>(w, gid, nb, raw[0]);
+    nn = take();
   }
-  for (int b = 0; b < nbat; ++b) {
-    const int nb = min(BATCH, total - b * BATCH);
+  for (int b = 0; nb > 0; ++b) {
     cp_async_wait_all();
     __syncthreads();
     stage_records<TILE, NT>(raw[b & 1], nb, ox, oy, gA, gB, gC);
     __syncthreads();
     stage_rowpairs<TILE, NT>(nb, gB, gC, rq);
     __syncthreads();
-    if (b + 1 < nbat) {
-      issue_records<NT, PF>(w, gid, min(BATCH, total - (b + 1) * BATCH), raw[(b + 1) & 1]);
-      if (b + 2 < nbat) keep(gid, src.next(gid));          // batch b + 2
+    int n2 = 0;
+    if (nn > 0) {
+      issue_records<NT, PF>(w, gid, nn, raw[(b + 1) & 1]);
+      n2 = take();
     }
     // Two operand sets in registers: Gaussian i + 1's loads overlap i's math.
     FwdOps<NQ> A, B;
@@ -1054,6 +1064,11 @@ __global__ void __launch_bounds__(TILE * TILE / BY) k_raster_fwd(Ws w, const uin
       fwd_gaussian<NQ>(acc, B, fcol);
     }
     __syncthreads();
+    nb = nn;
+    nn = n2;
+  }
+  if constexpr (GRID) {   // fewer found than counted: the list is incomplete
+    if (got < total && threadIdx.x == 0) atomicOr(&w.hdr->status, kStInternal);
   }
 
   const int H = D->out_h, W = D->out_w;
