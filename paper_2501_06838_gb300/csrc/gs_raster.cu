@@ -144,9 +144,9 @@ struct Candidates {
     hi = (uint32_t)(X1 & 0xffff) | ((uint32_t)Y1 << 16);
     seek(0);
   }
-  // this lane's k-th candidate from cur on (none: a window that meets nothing)
-  __device__ __forceinline__ uint2 load(int k) const {
-    return cur + 32 * k + (int)(threadIdx.x & 31) < total ? win[gid]
+  // the window of this lane's k-th candidate from cur on, g (none: one that meets nothing)
+  __device__ __forceinline__ uint2 load(int k, uint32_t g) const {
+    return cur + 32 * k + (int)(threadIdx.x & 31) < total ? win[g]
                                                           : make_uint2(0x7fff7fffu, 0x80008000u);
   }
   __device__ __forceinline__ void advance() {
@@ -185,9 +185,10 @@ struct GridSource {
 #pragma unroll
       for (int k = 0; k < KR; ++k) {
         g[k] = cand.gid;
-        v[k] = cand.load(k);
         cand.advance();
       }
+#pragma unroll
+      for (int k = 0; k < KR; ++k) v[k] = cand.load(k, g[k]);
 #pragma unroll
       for (int k = 0; k < KR; ++k) {
         const bool hit = cand.meets(v[k]);
@@ -209,6 +210,17 @@ struct GridSource {
     return nb;
   }
 };
+
+// A source's next batch as a call of its own, for the grid forward of tile 32:
+// inlined there, the candidate walk took the registers (168) that overlap the
+// operand loads with the arithmetic. Us, before that walk / inlined / as a call:
+// 5 images of 69 x 16 LR pixels, 4 Gaussians each, whole-image windows at scale 7
+// 853 / 957 / 843; 16 x 275, ratio window at 1.9 461 / 540 / 445; 256 x 256, 1
+// each, at 4 87 / 93 / 87. Tile 8 keeps it inline (as a call 49 -> 54, 55 -> 82).
+template <class Source, int PF>
+__device__ __noinline__ int next_apart(Source& src, uint32_t (&gid)[PF]) {
+  return src.next(gid);
+}
 
 // The candidate box of the pixel region [X0, X1] x [Y0, Y1] in grid mode (see
 // GridSource). A Gaussian of column j meets it only if s j - DL < x0 <= X1 and
@@ -833,7 +845,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 0) k_raster_fwd_team(Ws
     for (c.seek(c0); c.cur < c.total; c.cur += 128) {
       uint2 v[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) { v[k] = c.load(k); c.advance(); }
+      for (int k = 0; k < 4; ++k) { v[k] = c.load(k, c.gid); c.advance(); }
 #pragma unroll
       for (int k = 0; k < 4; ++k) cnt += __popc(__ballot_sync(0xffffffffu, c.meets(v[k])));
     }
@@ -855,7 +867,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 0) k_raster_fwd_team(Ws
         uint2 v[4];
         uint32_t g[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { g[k] = c.gid; v[k] = c.load(k); c.advance(); }
+        for (int k = 0; k < 4; ++k) { g[k] = c.gid; v[k] = c.load(k, c.gid); c.advance(); }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const bool hit = c.meets(v[k]);
@@ -1019,7 +1031,7 @@ __global__ void __launch_bounds__(TILE * TILE / BY) k_raster_fwd(Ws w, const uin
   uint32_t gid[PF];
   auto take = [&]() -> int {
     if (got >= total) return 0;
-    const int n = src.next(gid);
+    const int n = GRID && TILE == 32 ? next_apart(src, gid) : src.next(gid);
     if constexpr (GRID) {
       if (got + n > lcount) {   // the footprint count and the tile test disagree
         if (threadIdx.x == 0) atomicOr(&w.hdr->status, kStInternal);
@@ -1130,7 +1142,7 @@ struct PairSource {
 #pragma unroll
       for (int k = 0; k < KR; ++k) {
         g[k] = cand.gid;
-        v[k] = cand.load(k);
+        v[k] = cand.load(k, cand.gid);
         cand.advance();
       }
 #pragma unroll
