@@ -19,6 +19,7 @@ namespace {
 
 constexpr int kTopThreads = 1024;
 constexpr int kSumParts = 1024;   // block counts that every emit block adds up itself
+constexpr uint32_t kWideTiles = 32;   // tiles per Gaussian from which emit takes them one by one
 
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
@@ -53,7 +54,10 @@ __global__ void __launch_bounds__(kTopThreads) k_scan_top(unsigned long long* pa
 // then writes its Gaussians' pairs 32 at a time, each lane finding the Gaussian
 // its pair belongs to in the scanned counts (a warp's Gaussians one after the
 // other left most lanes idle: 3.7 pairs each on 100,000 Gaussians, 14.5 us; now
-// 8.6, and 34.4 -> 11.1 on 400,000).
+// 8.6, and 34.4 -> 11.1 on 400,000). A warp whose rectangles average more than
+// kWideTiles tiles has full lanes either way and spares itself the search: us on
+// 3,000 Gaussians, by pairs / by Gaussians: 11 tiles each 9 / 13, 21 11 / 13, 49
+// 18 / 14, 163 44 / 20, 950 225 / 49.
 // SUM: the partials are not scanned; every block adds them up itself, which
 // for up to kSumParts of them is less than a scan's launch (6 us).
 template <bool SUM>
@@ -95,6 +99,23 @@ __global__ void __launch_bounds__(kFootprintBlock) k_emit(Ws w) {
   const uint32_t end = off - start + cnt;                    // past the lane's last, from there
   const uint32_t total = __shfl_sync(0xffffffffu, end, 31);
   const uint32_t g0 = (uint32_t)(gi - lane);
+  if (total > 32u * kWideTiles) {   // large rectangles: one Gaussian's pairs at a time
+    for (int j = 0; j < 32; ++j) {
+      const uint32_t c = __shfl_sync(0xffffffffu, cnt, j);
+      if (c == 0u) continue;
+      const uint32_t at = start + __shfl_sync(0xffffffffu, end, j) - c;
+      const uint32_t key0 = __shfl_sync(0xffffffffu, tr.x, j);
+      const uint32_t tx = __shfl_sync(0xffffffffu, tr.y, j);
+      const uint32_t tw = __shfl_sync(0xffffffffu, tr.z, j);
+#pragma unroll 4
+      for (uint32_t i = lane; i < c; i += 32u) {
+        const uint32_t r = i / tw, q = i - r * tw;
+        w.keys[0][at + i] = key0 + r * tx + q;
+        w.vals[0][at + i] = g0 + (uint32_t)j;
+      }
+    }
+    return;
+  }
   for (uint32_t k0 = 0; k0 < total; k0 += 32u) {   // uniform over the warp
     const uint32_t k = min(k0 + lane, total - 1u);
     int j = 0;   // the first lane whose last pair is past k
