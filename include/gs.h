@@ -228,11 +228,28 @@ typedef struct gs_stats {
                            (GS_ADJOINT_TILE, _GAUSSIAN or _QUADRANT) */
 } gs_stats;
 
+/* How a call lays its work out, as gs_query_layout finds it. */
+typedef struct gs_layout {
+  int32_t raster;        /* forward: GS_RASTER_TILE or GS_RASTER_PAIR */
+  int32_t team;          /* forward: warps that share a tile's list (tile 16), 1: one warp */
+  int32_t adjoint;       /* GS_ADJOINT_TILE, _GAUSSIAN or _QUADRANT */
+  int32_t adjoint_parts; /* TILE and QUADRANT: parts each tile's list is cut into; else 1 */
+  int32_t block_x;       /* GAUSSIAN, every image on a reference grid: LR cells per block, */
+  int32_t block_y;       /*   else 0 */
+  int32_t reserved[2];
+} gs_layout;
+
 /* Bytes of workspace for rendering n_images images (arrays of n_images entries,
  * host memory) with room for `pair_capacity` (tile, Gaussian) pairs. Returns 0
  * when the arguments are invalid (see gs_last_error). Host-only, no CUDA call. */
 size_t gs_workspace_size(int32_t n_images, const gs_gaussians* g, const gs_view* v,
                          int64_t pair_capacity);
+
+/* The layout that the forward and the adjoint of these images take in a workspace
+ * of ws_bytes. Launches nothing and reads no device memory; adjoint_parts follows
+ * from the occupancy of the current device (1 where there is none). */
+gs_status gs_query_layout(int32_t n_images, const gs_gaussians* g, const gs_view* v,
+                          size_t ws_bytes, gs_layout* out);
 
 /* Exact number of (tile, Gaussian) pairs the render of these images emits.
  * Runs a counting pass over the Gaussians' windows on `stream` inside

@@ -23,7 +23,7 @@ GS_ADJOINT_AUTO, GS_ADJOINT_TILE, GS_ADJOINT_GAUSSIAN, GS_ADJOINT_QUADRANT = 0, 
 GS_BINNING_AUTO, GS_BINNING_SORT, GS_BINNING_GRID = 0, 1, 2
 GS_RASTER_AUTO, GS_RASTER_TILE, GS_RASTER_PAIR = 0, 1, 2
 
-EXPORTS = ("gs_workspace_size", "gs_count_pairs", "gs_render_fwd", "gs_render_bwd",
+EXPORTS = ("gs_workspace_size", "gs_query_layout", "gs_count_pairs", "gs_render_fwd", "gs_render_bwd",
            "gs_render_batched", "gs_render_batched_bwd", "gs_sync_status", "gs_read_stats",
            "gs_last_error", "gs_status_string", "gs_launch_count", "gs_timing_enable",
            "gs_timing_read", "gs_timing_release", "gs_kernel_name", "gs_version",
@@ -60,6 +60,12 @@ class GsStats(ctypes.Structure):
                 ("capacity", ctypes.c_int64), ("n_gaussians", ctypes.c_int64),
                 ("n_tiles", ctypes.c_int32), ("status", ctypes.c_int32),
                 ("raster", ctypes.c_int32), ("adjoint", ctypes.c_int32)]
+
+
+class GsLayout(ctypes.Structure):
+    _fields_ = [("raster", ctypes.c_int32), ("team", ctypes.c_int32), ("adjoint", ctypes.c_int32),
+                ("adjoint_parts", ctypes.c_int32), ("block_x", ctypes.c_int32),
+                ("block_y", ctypes.c_int32), ("reserved", ctypes.c_int32 * 2)]
 
 
 class GsPeaks(ctypes.Structure):
@@ -104,6 +110,7 @@ def load(path: str | None = None):
         fpp = ctypes.POINTER(ctypes.c_void_p)
         sig = {
             "gs_workspace_size": (sz, [i32, G, V, i64]),
+            "gs_query_layout": (i32, [i32, G, V, sz, ctypes.POINTER(GsLayout)]),
             "gs_count_pairs": (i32, [i32, G, V, vp, sz, vp, ctypes.POINTER(i64)]),
             "gs_render_fwd": (i32, [G, V, vp, vp, sz, vp]),
             "gs_render_bwd": (i32, [G, V, vp, vp, vp, sz, vp]),

@@ -445,39 +445,39 @@ int32_t list_parts(int64_t tiles, int64_t full) {
   return 2 * tiles > full ? 1 : (int32_t)std::min<int64_t>(kBwdParts, (2 * full + tiles - 1) / tiles);
 }
 
-// The tile adjoint: a persistent launch of one-warp CTAs.
-cudaError_t launch_tile(void (*whole)(Ws, const uint32_t*), void (*split)(Ws, const uint32_t*), Ws w,
-                        const uint32_t* lists, cudaStream_t s) {
-  const int64_t full = resident_grid((const void*)whole, 32, INT32_MAX);
-  w.bwd_parts = list_parts(w.tiles, full);
-  if (w.bwd_parts == 1)
-    return launch_chain(whole, dim3((unsigned)std::min<int64_t>(full, w.tiles)), dim3(32), 0, s, w, lists);
-  const int64_t ctas = resident_grid((const void*)split, 32, (int64_t)w.tiles * w.bwd_parts);
-  return launch_chain(split, dim3((unsigned)ctas), dim3(32), 0, s, w, lists);
-}
+using BwdKernel = void (*)(Ws, const uint32_t*);
 
-// The quadrant adjoint: a CTA per tile, or per part of a tile's list.
-cudaError_t launch_quad(Ws w, const uint32_t* lists, cudaStream_t s) {
-  const dim3 block(32 * kBwWarps);
-  w.bwd_parts = list_parts(w.tiles, resident_grid((const void*)k_raster_bwd_quad<false>,
-                                                  32 * kBwWarps, INT32_MAX));
-  const dim3 grid((unsigned)((int64_t)w.tiles * w.bwd_parts));
-  if (w.bwd_parts == 1) return launch_chain(k_raster_bwd_quad<false>, grid, block, 0, s, w, lists);
-  return launch_chain(k_raster_bwd_quad<true>, grid, block, 0, s, w, lists);
+// The tile adjoint's kernels over whole lists and over parts.
+BwdKernel tile_kernel(int tile, bool split) {
+  switch (tile) {
+    case 8: return split ? k_raster_bwd_tile<8, true> : k_raster_bwd_tile<8, false>;
+    case 32: return split ? k_raster_bwd_tile<32, true> : k_raster_bwd_tile<32, false>;
+    default: return split ? k_raster_bwd_tile<16, true> : k_raster_bwd_tile<16, false>;
+  }
 }
 
 }  // namespace
 
-cudaError_t launch_raster_bwd_tile(const Ws& w, const uint32_t* lists, bool quadrants,
+int32_t raster_bwd_parts(const Ws& w, bool quadrants) {
+  const BwdKernel whole = quadrants ? k_raster_bwd_quad<false> : tile_kernel(w.tile, false);
+  return list_parts(w.tiles, resident_grid((const void*)whole, quadrants ? 32 * kBwWarps : 32, INT32_MAX));
+}
+
+cudaError_t launch_raster_bwd_tile(const Ws& ws, const uint32_t* lists, bool quadrants,
                                    cudaStream_t s) {
-  if (w.tiles == 0) return cudaSuccess;
+  if (ws.tiles == 0) return cudaSuccess;
   LaunchScope ls(kKRasterBwd, s);
-  if (quadrants) return launch_quad(w, lists, s);   // tile 16 (the caller checks)
-  switch (w.tile) {
-    case 8: return launch_tile(k_raster_bwd_tile<8, false>, k_raster_bwd_tile<8, true>, w, lists, s);
-    case 32: return launch_tile(k_raster_bwd_tile<32, false>, k_raster_bwd_tile<32, true>, w, lists, s);
-    default: return launch_tile(k_raster_bwd_tile<16, false>, k_raster_bwd_tile<16, true>, w, lists, s);
-  }
+  Ws w = ws;
+  w.bwd_parts = raster_bwd_parts(w, quadrants);
+  const bool split = w.bwd_parts > 1;
+  const int64_t units = (int64_t)w.tiles * w.bwd_parts;
+  if (quadrants)   // tile 16 (the caller checks): a CTA per tile, or per part of a tile's list
+    return launch_chain(split ? k_raster_bwd_quad<true> : k_raster_bwd_quad<false>,
+                        dim3((unsigned)units), dim3(32 * kBwWarps), 0, s, w, lists);
+  // a persistent launch of one-warp CTAs
+  const BwdKernel kernel = tile_kernel(w.tile, split);
+  return launch_chain(kernel, dim3((unsigned)resident_grid((const void*)kernel, 32, units)), dim3(32),
+                      0, s, w, lists);
 }
 
 }  // namespace gs

@@ -680,6 +680,31 @@ size_t gs_workspace_size(int32_t n_images, const gs_gaussians* g, const gs_view*
   return make_layout(n_images, P.n, P.tiles, pair_capacity, P.grid).total;
 }
 
+gs_status gs_query_layout(int32_t n_images, const gs_gaussians* g, const gs_view* v,
+                          size_t ws_bytes, gs_layout* out) {
+  if (!out) return fail(GS_ERR_INVALID, "null layout");
+  Call c;
+  // the workspace's address is not used: the smallest that is aligned
+  gs_status st = prepare(n_images, g, v, reinterpret_cast<void*>(uintptr_t(256)), ws_bytes, &c);
+  if (st != GS_OK) return st;
+  std::memset(out, 0, sizeof(*out));
+  out->raster = c.w.pair ? GS_RASTER_PAIR : GS_RASTER_TILE;
+  out->team = c.w.team ? c.w.team : 1;
+  out->adjoint = c.P.adjoint;
+  out->adjoint_parts = 1;
+  if (c.P.adjoint != GS_ADJOINT_GAUSSIAN) {
+    int devices = 0;
+    if (cudaGetDeviceCount(&devices) == cudaSuccess && devices > 0)
+      out->adjoint_parts = raster_bwd_parts(c.w, c.P.adjoint == GS_ADJOINT_QUADRANT);
+    else
+      cudaGetLastError();
+  } else if (c.w.n_gblocks > 0) {
+    out->block_x = c.w.gb_x;
+    out->block_y = c.w.gb_y;
+  }
+  return GS_OK;
+}
+
 gs_status gs_count_pairs(int32_t n_images, const gs_gaussians* g, const gs_view* v, void* ws,
                          size_t ws_bytes, void* stream, int64_t* pairs_out) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);

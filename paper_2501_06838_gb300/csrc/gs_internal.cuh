@@ -245,6 +245,7 @@ cudaError_t launch_raster_bwd_gblock(const Ws& w, cudaStream_t s);   // needs w.
 // with the Gaussians of the tile's list whose window meets it
 cudaError_t launch_raster_bwd_tile(const Ws& w, const uint32_t* lists, bool quadrants,
                                    cudaStream_t s);
+int32_t raster_bwd_parts(const Ws& w, bool quadrants);   // parts of each list it cuts (host only)
 
 // Kernel ids for launch accounting / per-kernel timing.
 enum KernelId {

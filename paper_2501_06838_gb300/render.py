@@ -357,6 +357,16 @@ def read_stats(ws: Workspace, stream=None) -> dict:
     return {f: getattr(st, f) for f, _ in _abi.GsStats._fields_}
 
 
+def query_layout(gs, views, ws: Workspace, tile=0, batch=0) -> dict:
+    """The layout the forward and the adjoint of these images take in `ws`: raster
+    (TILE or PAIR), team (warps per tile), adjoint kind, adjoint_parts (of each
+    tile's list) and block_x, block_y (LR cells per block, GAUSSIAN adjoint)."""
+    n, G, V = _arrays(gs, views, tile, batch)
+    lo = _abi.GsLayout()
+    _abi.check(_abi.load().gs_query_layout(n, G, V, ws.nbytes, ctypes.byref(lo)), "gs_query_layout")
+    return {f: getattr(lo, f) for f, _ in _abi.GsLayout._fields_ if f != "reserved"}
+
+
 def launch_count() -> int:
     return int(_abi.load().gs_launch_count())
 

@@ -172,8 +172,8 @@ def test_pair_raster_equals_tile_raster(case, batch):
 
 def test_pair_raster_batched_bands_and_auto():
     """Pairs over an uneven batch (odd tile columns leave a last tile alone in
-    its pair), row bands of one image, and the AUTO choice (pairs only for
-    3-sigma windows at scale >= 6)."""
+    its pair), row bands of one image, and the AUTO choice (a batch of small
+    images with short lists keeps pairs from scale 6 on, one small image tiles)."""
     import paper_2501_06838_gb300 as gs
     gsets, views = [], []
     for i, (h, w, s) in enumerate([(20, 26, 2.7), (17, 23, 6.5), (9, 31, 12.0), (5, 5, 11.0)]):
@@ -186,7 +186,7 @@ def test_pair_raster_batched_bands_and_auto():
             v.binning, v.raster = GRID, raster
         o, ws = gs.render_batched(dgs, views, check=True)
         res[raster] = ([x.cpu().numpy() for x in o], gs.read_stats(ws)["raster"])
-    assert res[0][1] == RASTER_PAIR   # a scale >= 6 with 3-sigma windows
+    assert res[0][1] == RASTER_PAIR   # four small images, a scale >= 6, 3-sigma windows
     for a, b, c in zip(res[RASTER_TILE][0], res[RASTER_PAIR][0], res[0][0]):
         assert np.array_equal(a, b) and np.array_equal(a, c)
     for x, g, v in zip(res[RASTER_PAIR][0], gsets, views):

@@ -15,7 +15,8 @@ from paper_2501_06838_gb300 import _abi
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 STRUCTS = {"gs_head": _abi.GsHead, "gs_gaussians": _abi.GsGaussians, "gs_view": _abi.GsView,
-           "gs_stats": _abi.GsStats, "gs_peaks": _abi.GsPeaks, "gs_tuning": _abi.GsTuning}
+           "gs_stats": _abi.GsStats, "gs_peaks": _abi.GsPeaks, "gs_layout": _abi.GsLayout,
+           "gs_tuning": _abi.GsTuning}
 ENUMS = ["GS_OK", "GS_ERR_INVALID", "GS_ERR_CAPACITY", "GS_ERR_CUDA", "GS_ERR_UNSUPPORTED",
          "GS_ERR_TIMEOUT", "GS_ERR_INTERNAL", "GS_F32", "GS_BF16", "GS_F16", "GS_NORM_DENSITY",
          "GS_NORM_PEAK", "GS_WINDOW_SIGMA", "GS_WINDOW_RATIO", "GS_ALIGN_EQ4", "GS_ALIGN_HALF",

@@ -26,9 +26,10 @@ CASES = {
     "sparse_sigma": (20, 24, 4, dict(scale=4.6)),        # 45 Gaussians per tile: lists below a segment
     "thin_sigma": (24, 24, 1, dict(scale=4.0)),          # 16 per tile, lists of about 75
     "wide_sigma": (11, 14, 4, dict(scale=12.0)),         # 6 per tile, lists of about 130
-    "many_tiles_sigma": (112, 113, 9, dict(scale=4.0)),  # 783 tiles, 145 per tile: one warp
+    "many_tiles_sigma": (112, 113, 9, dict(scale=4.0)),  # 812 tiles, 140 per tile: one warp
     "many_tiles_team": (150, 151, 9, dict(scale=3.0)),   # 841 tiles, 242 per tile: teams again
 }
+TEAM = {"ratio_many_tiles": 4, "many_tiles_sigma": 1, "many_tiles_team": 4}   # the others: 8 warps
 
 
 def _scene(case):
@@ -46,17 +47,20 @@ def test_teams_equal_other_layouts(case):
     dg = device_gaussians(g)
     imgs, grads = [], []
     go = torch.from_numpy(S.grad_out(3, v.out_h, v.out_w)).cuda()
-    for binning, raster in ((GRID, TILE), (SORT, TILE), (GRID, PAIR)):
+    # batch 64: one warp per tile; pairs whose segments may end in the second half of a batch
+    for binning, raster, batch in ((GRID, TILE, 0), (SORT, TILE, 0), (GRID, PAIR, 0), (GRID, TILE, 64),
+                                   (GRID, PAIR, 64)):
         v.binning, v.raster = binning, raster
-        out, ws = gs.render(dg, v, check=True)
+        out, ws = gs.render(dg, v, batch=batch, check=True)
         assert gs.read_stats(ws)["raster"] == raster
+        layout = gs.query_layout([dg], [v], ws, batch=batch)
+        assert layout["raster"] == raster
+        assert layout["team"] == (1 if raster == PAIR or batch else TEAM.get(case, 8))
         imgs.append(out.cpu().numpy())
         # the list each route leaves for the adjoint
-        grads.append(gs.render_bwd(dg, v, go, ws, check=True).cpu().double().numpy())
-    v.binning, v.raster = GRID, TILE
-    out64, _ = gs.render(dg, v, batch=64, check=True)   # batch 64: one warp per tile
-    assert np.array_equal(imgs[0], imgs[1]) and np.array_equal(imgs[0], imgs[2])
-    assert np.array_equal(imgs[0], out64.cpu().numpy())
+        grads.append(gs.render_bwd(dg, v, go, ws, batch=batch, check=True).cpu().double().numpy())
+    for im in imgs[1:]:
+        assert np.array_equal(imgs[0], im)
     assert np.all(normwise(imgs[0].astype(np.float64), oracle.render(g, v), axis=(1, 2)) < 1e-5)
     ref = oracle.adjoint(g, v, go.cpu().numpy())
     for gr in grads:
@@ -68,12 +72,14 @@ def test_team_image_alone_and_in_a_batch():
     whether teams run) nor on the pair capacity (a team enumerates its list
     itself when it does not fit)."""
     import paper_2501_06838_gb300 as gs
-    g, v = _scene("dense_sigma")
+    g, v = _scene("dense_sigma")   # a team alone, not in the batch
     big = S.draw_gaussians(5, 200, 180, 1, (0.3, 2.0))
     bv = S.View(200, 180, 1000, 900, 5.0)
     dg, db = device_gaussians(g), device_gaussians(big)
-    alone, _ = gs.render(dg, v, check=True)
-    (together, _), _ = gs.render_batched([dg, db], [v, bv], check=True)
+    alone, ws = gs.render(dg, v, check=True)
+    assert gs.query_layout([dg], [v], ws)["team"] == 8
+    (together, _), ws = gs.render_batched([dg, db], [v, bv], check=True)
+    assert gs.query_layout([dg, db], [v, bv], ws)["team"] == 1
     assert np.array_equal(alone.cpu().numpy(), together.cpu().numpy())
     for case in ("dense_sigma", "whole_4608"):
         g, v = _scene(case)
