@@ -440,9 +440,24 @@ namespace {
 // lists of 4,000 to 10,000): 656 -> 86 us (parts that fill the chip once: 106).
 // A part stages the tile's gradient again and leaves a chunk short, so a fuller
 // chip keeps whole lists: 16 crops with short lists took 38.7 us in parts
-// against 37.1.
-int32_t list_parts(int64_t tiles, int64_t full) {
-  return 2 * tiles > full ? 1 : (int32_t)std::min<int64_t>(kBwdParts, (2 * full + tiles - 1) / tiles);
+// against 37.1. And a part costs a CTA whether or not it has a chunk, so a list
+// is cut into no more than one part per `entries` of the lists' mean length,
+// which the pair capacity bounds (sized by a count, it is the mean), or into as
+// many as make `spare` CTAs in all: those are next to free, and shorten what one
+// long list among short ones takes. Adjoint, us, whole lists / cut so / a chip's
+// worth of parts: tile 16, 256 tiles, lists of 16 9.7 / 10.4 / 16.3, 62 19.2 / 12.7
+// / 18.7, 125 33.5 / 16.4 / 21.7; 1,024 tiles, 16 12.1 / 12.1 / 21.2, 64 27.6 / 25.3
+// / 26.5; 2,025 tiles, 16 15.6 / 15.6 / 24.7, 64 42.8 / 30.1 / 31.3; quadrants, 256
+// tiles, 63 9.4 / 9.4 / 10.3, 250 16.0 / 14.8 / 15.6. With half the Gaussians in a
+// 25th of the tiles: tile 16, 64 tiles, mean 14 26.1 / 9.6 / 10.4, 256 tiles, 62 132
+// / 41 / 19; quadrants, 256 tiles, 62 27.8 / 12.7 / 10.7.
+int32_t list_parts(const Ws& w, int64_t full, int64_t entries, int64_t spare) {
+  const int64_t tiles = w.tiles;
+  if (2 * tiles > full) return 1;
+  const int64_t fill = std::min<int64_t>(kBwdParts, (2 * full + tiles - 1) / tiles);
+  const int64_t mean = w.capacity / tiles;
+  const int64_t worth = std::max((mean + entries / 2) / entries, spare / tiles);
+  return (int32_t)std::max<int64_t>(1, std::min(fill, worth));
 }
 
 using BwdKernel = void (*)(Ws, const uint32_t*);
@@ -459,8 +474,12 @@ BwdKernel tile_kernel(int tile, bool split) {
 }  // namespace
 
 int32_t raster_bwd_parts(const Ws& w, bool quadrants) {
-  const BwdKernel whole = quadrants ? k_raster_bwd_quad<false> : tile_kernel(w.tile, false);
-  return list_parts(w.tiles, resident_grid((const void*)whole, quadrants ? 32 * kBwWarps : 32, INT32_MAX));
+  // a chunk of a quadrant CTA is four warps', one of an 8 x 8 tile a quarter of the work
+  if (quadrants)
+    return list_parts(w, resident_grid((const void*)k_raster_bwd_quad<false>, 32 * kBwWarps, INT32_MAX),
+                      64, 1024);
+  return list_parts(w, resident_grid((const void*)tile_kernel(w.tile, false), 32, INT32_MAX),
+                    w.tile == 8 ? 64 : 16, 512);
 }
 
 cudaError_t launch_raster_bwd_tile(const Ws& ws, const uint32_t* lists, bool quadrants,

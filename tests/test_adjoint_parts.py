@@ -33,3 +33,32 @@ def test_split_lists(n, mode, tile):
     got = gs.render_bwd(dg, v, torch.from_numpy(go).cuda(), ws, tile=tile, check=True)
     err = normwise(got.cpu().double().numpy(), oracle.adjoint(g, v, go), axis=0)
     assert np.all(err < 1e-5), err
+
+
+@pytest.mark.parametrize("mode,tile,edge,longest,whole", [(TILE, 8, 30, 95, 1), (TILE, 16, 30, 23, 1),
+                                                          (TILE, 32, 30, 23, 1), (QUADRANT, 16, 20, 159, 2)])
+def test_short_lists_stay_whole(mode, tile, edge, longest, whole):
+    """A part costs a CTA, so short lists are not cut for the chip's sake, or only
+    as far as the CTAs are next to free; a larger workspace (whose capacity no
+    longer tells the mean length) has them cut, with the same gradients to
+    rounding."""
+    import torch
+    import paper_2501_06838_gb300 as gs
+    rng = np.random.default_rng(tile)
+    side = edge * tile
+    n = edge * edge * longest // 3
+    g = absolute(rng.uniform(0, side - 1, (n, 2)), rng.uniform(0.3, 0.6, (n, 2)), rng.uniform(-0.9, 0.9, n),
+                 rng.uniform(0.1, 1, (n, 3)), rng.uniform(0.1, 1, n), side, side)
+    v = S.View(side, side, side, side, 1.0)
+    v.adjoint = mode
+    dg, go = device_gaussians(g), torch.from_numpy(S.grad_out(tile, side, side)).cuda()
+    pairs = gs.count_pairs([dg], [v], tile=tile)
+    assert pairs < edge * edge * longest
+    ref = oracle.adjoint(g, v, go.cpu().numpy())
+    for capacity in (pairs, 40 * pairs):
+        ws = gs.make_workspace([dg], [v], capacity, tile=tile)
+        parts = gs.query_layout([dg], [v], ws, tile=tile)["adjoint_parts"]
+        assert parts == whole if capacity == pairs else parts > whole
+        gs.render(dg, v, ws=ws, tile=tile, check=True)
+        got = gs.render_bwd(dg, v, go, ws, tile=tile, check=True).cpu().double().numpy()
+        assert np.all(normwise(got, ref, axis=0) < 1e-5)
