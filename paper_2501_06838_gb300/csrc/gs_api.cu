@@ -340,24 +340,64 @@ int team_of(const Problem& P, const gs_gaussians* g, const gs_view* v) {
 // LR cells per block of the block Gaussian-warp adjoint. A block shares the
 // copied box of upstream gradient, so large blocks pay the windows' halo less
 // often, until the box no longer fits shared memory (then its Gaussians only
-// share L1) or the blocks are too few and too uneven to fill the chip. Measured,
-// us, 8 x 8 / 8 x 4 / 4 x 4 / 4 x 2 cells, one Gaussian per cell with sigma up to
-// 2: scale 4 75.6 / 81.2 / 97.5 / 127, 5 66.3 / 56.9 / 63.5 / 81.7, 6 68.5 / 60.8
-// / 51.3 / 62.1, 12 154 / 95.9 / 65.3 / 70.3; four per cell at scale 8 258 / 231
-// / 191 / 186; sixteen at scale 2 174 / 152 / 120 / 107; whole-image windows at
-// scale 3 569 / 291 / 162 / 160.
-void gblock_shape(int32_t n_images, const gs_gaussians* g, const gs_view* v, int32_t* x, int32_t* y) {
+// share L1) or the blocks are too few and too uneven to fill the chip (two CTAs
+// per SM). All figures: us, 8 x 8 / 8 x 4 / 4 x 4 / 4 x 2 cells.
+//   Few blocks (of 8 x 8; less than 1.2 rounds of the chip with one Gaussian per
+// cell, 3.5 with more): the scale says how large the windows are. 120 x 120 cells,
+// sigma up to 2: scale 4.2 26 / 27 / 27 / 33, 5 36 / 32 / 32 / 38, 6 50 / 45 / 37 /
+// 44, 12 145 / 140 / 131 / 139; four per cell, 64 x 64, scale 4 57 / 34 / 26 / 28;
+// sixteen, scale 2 139 / 74 / 49 / 49; 60 x 80, whole-image windows at scale 2
+// 322 / 175 / 94 / 95.
+//   Many blocks: the largest whose box is likely to fit, from the windows' size.
+// That is known from the views, or (k-sigma boxes) the mean side follows from the
+// pairs per Gaussian, which the pair capacity bounds; the largest windows of a
+// block are some 3 times the mean. Lines by measurement on 30,450 to 2,101,120
+// Gaussians: no choice was slower than 8 x 8 by more than 7%. One per cell, 243 x
+// 429, scale 6, sigma up to 1 104 / 115 / 144 / 193, 2 205 / 200 / 225 /
+// 301, 3 343 / 362 / 404 / 484 (fits no shape); scale 8, sigma up to 1 183 / 146 /
+// 179 / 238; 150 x 203, scale 5, sigma up to 2 60 / 53 / 61 / 78 (from 1,200 blocks
+// on such a box takes 8 x 8: 129 / 132); ratio window 0.02 at scale 7 124 / 92 / 91
+// / 106; four per cell, 280 x 469, scale 1.2, sigma up to 0.8 273 / 280 / 298 / 335,
+// scale 6, sigma up to 2 901 / 909 / 752 / 881.
+void gblock_shape(const Problem& P, const gs_gaussians* g, const gs_view* v, int64_t capacity,
+                  int32_t* x, int32_t* y) {
   float scale = 0.0f;
   int m = 0;
-  bool boxes = true;   // every window a k-sigma box
-  for (int i = 0; i < n_images; ++i) {
-    scale = std::max(scale, v[i].scale);
+  int64_t blocks = 0;   // of 8 x 8 cells
+  bool boxes = true;    // every window a k-sigma box
+  double wx = 0.0, wy = 0.0;   // the other windows' sides, HR px
+  for (int i = 0; i < P.n_images; ++i) {
+    const gs_view& V = v[i];
+    scale = std::max(scale, V.scale);
     m = std::max(m, (int)g[i].ref_grid_m);
-    if (v[i].window != GS_WINDOW_SIGMA || !(v[i].trunc_k > 0.0f)) boxes = false;
+    blocks += (int64_t)((V.lr_h + 7) / 8) * ((V.lr_w + 7) / 8);
+    if (V.window == GS_WINDOW_SIGMA && V.trunc_k > 0.0f) continue;
+    boxes = false;
+    const double r = V.trunc_k > 0.0f ? 2.0 * (double)V.scale * (double)V.trunc_k : HUGE_VAL;
+    wx = std::max(wx, std::min((double)V.out_w, r * V.lr_w));
+    wy = std::max(wy, std::min((double)V.out_h, r * V.lr_h));
   }
-  const bool small = boxes && m <= 1;
-  *x = small && scale < 5.75f ? 8 : 4;
-  *y = small && scale < 4.5f ? 8 : m >= 16 ? 2 : 4;
+  const bool one = m <= 1;
+  if (blocks < (one ? 365 : 1065)) {
+    *x = boxes && one && scale < 5.75f ? 8 : 4;
+    *y = boxes && one && scale < 4.5f ? 8 : m >= 16 ? 2 : 4;
+    return;
+  }
+  if (boxes) {   // a window of side w meets (w / tile + 1)^2 tiles on average
+    const double pairs = std::max(1.0, (double)capacity / (double)std::max<int64_t>(1, P.n));
+    wx = wy = 3.2 * P.tile * (std::sqrt(pairs) - 1.0);
+  }
+  auto floats = [&](int gx, int gy) { return 3.0 * (gx * (double)scale + wx) * (gy * (double)scale + wy); };
+  *x = 8;
+  *y = 8;
+  if (one) {
+    if (floats(8, 8) <= (boxes ? (blocks < 1200 ? 36e3 : 38e3) : 22e3)) return;
+    if (floats(8, 4) <= (boxes ? 46e3 : 23.5e3)) *y = 4;
+    else if (!boxes) *x = *y = 4;
+  } else {
+    *y = 4;
+    if (floats(8, 4) > (boxes ? 27e3 : 23.5e3) && (!boxes || floats(4, 4) <= 46e3)) *x = 4;
+  }
 }
 
 struct Call {
@@ -423,7 +463,7 @@ gs_status prepare(int32_t n_images, const gs_gaussians* g, const gs_view* v, voi
   w.adjoint = c->P.adjoint;
   // blocks of LR cells (the Gaussian-warp adjoint's block form), when
   // every image's Gaussians sit on a reference grid
-  gblock_shape(n_images, g, v, &w.gb_x, &w.gb_y);
+  gblock_shape(c->P, g, v, cap, &w.gb_x, &w.gb_y);
   int64_t gblocks = 0;
   for (int i = 0; i < n_images; ++i) {
     if (g[i].ref_grid_m == 0) { gblocks = 0; break; }
