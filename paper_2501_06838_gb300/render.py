@@ -21,6 +21,7 @@ from __future__ import annotations
 import ctypes
 import dataclasses
 import math
+import operator
 from typing import Sequence
 
 import torch
@@ -399,6 +400,17 @@ class GSRender(torch.autograd.Function):
         return (*_split_grads(gr, ctx.g.offset.dtype), None, None, None)
 
 
+def _cut(ts, sizes):
+    """Consecutive rows of every tensor, sizes[i] for image i (fewer where a tensor
+    ends: slices)."""
+    sizes = [operator.index(n) for n in sizes]
+    total = sum(sizes)
+    if min(sizes, default=0) >= 0 and all(t.shape[0] >= total for t in ts):
+        return [t[:total].split(sizes) for t in ts]   # one call per tensor instead of one per image
+    ends = [sum(sizes[:i]) for i in range(len(sizes) + 1)]
+    return [[t[a:b] for a, b in zip(ends, ends[1:])] for t in ts]
+
+
 class GSRenderBatched(torch.autograd.Function):
     """Images of uneven sizes and scales in one launch chain. Parameters are
     concatenated over images; sizes[i] Gaussians belong to image i. With a
@@ -408,8 +420,7 @@ class GSRenderBatched(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, views, ref_grid_m, sizes, head, offset, sigma, rho, rgb, alpha):
-        sizes, n = list(sizes), sum(sizes)
-        ts = [t.contiguous()[:n].split(sizes) for t in (offset, sigma, rho, rgb, alpha)]
+        ts = _cut([t.contiguous() for t in (offset, sigma, rho, rgb, alpha)], sizes)
         gs = [Gaussians(*t, ref_grid_m=ref_grid_m, head=head) for t in zip(*ts)]
         outs, ws = render_batched(gs, views)
         ctx.gs, ctx.views, ctx.ws, ctx.dtype = gs, views, ws, offset.dtype
