@@ -180,12 +180,13 @@ def _arrays(gs: Sequence[Gaussians], views, tile=0, batch=0):
     n = len(gs)
     if n != len(views) or n == 0:
         raise ValueError("need one view per image and at least one image")
+    owners = [g.head for g in gs]   # held: while they live, an id names one of them
     heads = {}   # one struct per head object of this call
-    for g in gs:
-        if g.head is not None and id(g.head) not in heads:
-            heads[id(g.head)] = _head_struct(g.head)
+    for h in owners:
+        if h is not None and id(h) not in heads:
+            heads[id(h)] = _head_struct(h)
     # (a ctypes array takes a tuple of fields per element)
-    G = (_abi.GsGaussians * n)(*[_fields_g(g, heads.get(id(g.head))) for g in gs])
+    G = (_abi.GsGaussians * n)(*[_fields_g(g, heads.get(id(h))) for g, h in zip(gs, owners)])
     G._head_keep = list(heads.values())   # head structs the array points to
     V = (_abi.GsView * n)(*[_fields_v(v, tile, batch) for v in views])
     return n, G, V
