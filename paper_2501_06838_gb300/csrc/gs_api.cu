@@ -53,7 +53,7 @@ cudaEvent_t take_event() {
 }
 
 const char* kKernelNames[kKNumKernels] = {
-    "setup",      "preprocess",    "reserved",      "scan_top",   "radix_rowscan",
+    "setup",      "preprocess",    "count",         "scan_top",   "radix_rowscan",
     "emit",       "radix_hist",    "radix_scatter", "ranges",     "raster_fwd",
     "raster_bwd", "preprocess_bwd", "reserved12",    "raster_bwd_gw"};
 

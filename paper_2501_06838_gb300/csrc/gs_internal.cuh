@@ -249,7 +249,7 @@ int32_t raster_bwd_parts(const Ws& w, bool quadrants);   // parts of each list i
 
 // Kernel ids for launch accounting / per-kernel timing.
 enum KernelId {
-  kKSetup = 0, kKPreprocess, kKReserved2, kKScanTop, kKRadixRowscan, kKEmit, kKRadixHist,
+  kKSetup = 0, kKPreprocess, kKCount, kKScanTop, kKRadixRowscan, kKEmit, kKRadixHist,
   kKRadixScatter, kKRanges, kKRasterFwd, kKRasterBwd, kKPreprocessBwd, kKReserved12, kKRasterBwdGw,
   kKNumKernels
 };

@@ -673,7 +673,7 @@ cudaError_t launch_preprocess(const Ws& w, const ImageDesc& first, cudaStream_t 
 
 cudaError_t launch_count(const Ws& w, cudaStream_t s) {
   if (w.n == 0) return cudaSuccess;
-  LaunchScope ls(kKPreprocess, s);
+  LaunchScope ls(kKCount, s);
   const int64_t blocks = (w.n + kFootprintBlock - 1) / kFootprintBlock;
   return launch_chain(k_count, dim3((unsigned)blocks), dim3(kFootprintBlock), 0, s, w);
 }

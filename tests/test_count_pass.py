@@ -71,3 +71,21 @@ def test_count_batch_band_and_status():
     with pytest.raises(gs.GsError) as ei:
         gs.count_pairs([device_gaussians(bad)], [views[names.index("f32_m1")]])
     assert ei.value.status == 1
+
+
+def test_count_is_timed_as_itself():
+    """Per-kernel times: the counting pass under its own name, not the footprint pass's."""
+    import paper_2501_06838_gb300 as gs
+    g, kw = CASES["f32_m1"]
+    dg, v = device_gaussians(g), _view(g, **kw)
+    gs.timing_read()
+    gs.timing_enable()
+    try:
+        gs.count_pairs([dg], [v])
+        counted = gs.timing_read()
+        gs.render(dg, v, check=True)   # counts, then renders
+        rendered = gs.timing_read()
+    finally:
+        gs.timing_enable([])
+    assert {k: n for k, (_, n) in counted.items()} == {"setup": 1, "count": 1}
+    assert {k: n for k, (_, n) in rendered.items()} == {"setup": 2, "count": 1, "preprocess": 1, "raster_fwd": 1}
