@@ -129,6 +129,8 @@ struct Candidates {
   int L, total, cur;     // candidates per row, in all, next to test
   uint32_t gid, wrap;    // this lane's candidate; from a row's end to the next row's start
   int col;               // its position in its row
+  int step;              // advance_flat: 32 candidates on, modulo whole rows
+  uint32_t jump;         // ... and in gids
   uint32_t lo, hi;       // the region: (X0, Y0) and (X1, Y1), output rows
   // to candidate `from` (lane 0's)
   __device__ __forceinline__ void seek(int from) {
@@ -140,6 +142,9 @@ struct Candidates {
   }
   __device__ __forceinline__ void start(int X0, int X1, int Y0, int Y1) {
     wrap = (uint32_t)(rstride - L);
+    const int rows = L > 0 ? 32 / L : 0;
+    step = 32 - rows * L;
+    jump = 32u + (uint32_t)rows * wrap;
     lo = (uint32_t)(X0 & 0xffff) | ((uint32_t)Y0 << 16);
     hi = (uint32_t)(X1 & 0xffff) | ((uint32_t)Y1 << 16);
     seek(0);
@@ -157,6 +162,15 @@ struct Candidates {
     } else if (L > 0) {
       while (col >= L) { col -= L; gid += wrap; }
     }
+  }
+  // the same without a branch, for tile 32: its tiles are few and their boxes, at a
+  // large scale, rows of a few cells that the loop above wraps one at a time (us:
+  // 5 images of 121 x 119 LR pixels at scale 18 392 -> 379, 178 x 203 at 23 301 ->
+  // 290; in the pair forward 913 -> 936 at 5760 x 3240, in tile 16's 48.6 -> 50)
+  __device__ __forceinline__ void advance_flat() {
+    col += step;
+    gid += jump;
+    if (col >= L) { col -= L; gid += wrap; }
   }
   // the window meets the region: x0 <= X1, y0 <= Y1, x1 >= X0, y1 >= Y0
   __device__ __forceinline__ bool meets(uint2 v) const {
@@ -185,7 +199,7 @@ struct GridSource {
 #pragma unroll
       for (int k = 0; k < KR; ++k) {
         g[k] = cand.gid;
-        cand.advance();
+        if constexpr (NT == 64 && PF == 1) cand.advance_flat(); else cand.advance();
       }
 #pragma unroll
       for (int k = 0; k < KR; ++k) v[k] = cand.load(k, g[k]);
@@ -211,12 +225,13 @@ struct GridSource {
   }
 };
 
-// A source's next batch as a call of its own, for the grid forward of tile 32:
-// inlined there, the candidate walk took the registers (168) that overlap the
-// operand loads with the arithmetic. Us, before that walk / inlined / as a call:
-// 5 images of 69 x 16 LR pixels, 4 Gaussians each, whole-image windows at scale 7
-// 853 / 957 / 843; 16 x 275, ratio window at 1.9 461 / 540 / 445; 256 x 256, 1
-// each, at 4 87 / 93 / 87. Tile 8 keeps it inline (as a call 49 -> 54, 55 -> 82).
+// A source's next batch as a call of its own, for the grid forward of tile 32 with
+// 64 Gaussians a round: inlined there, the candidate walk took the registers (168)
+// that overlap the operand loads with the arithmetic. Us, before that walk /
+// inlined / as a call: 5 images of 69 x 16 LR pixels, 4 Gaussians each,
+// whole-image windows at scale 7 853 / 957 / 843; 16 x 275, ratio window at 1.9
+// 461 / 540 / 445; 256 x 256, 1 each, at 4 87 / 93 / 87. Tile 8 and rounds of 128
+// keep it inline (as a call 49 -> 54, 55 -> 82; 478 -> 531).
 template <class Source, int PF>
 __device__ __noinline__ int next_apart(Source& src, uint32_t (&gid)[PF]) {
   return src.next(gid);
@@ -1031,7 +1046,7 @@ __global__ void __launch_bounds__(TILE * TILE / BY) k_raster_fwd(Ws w, const uin
   uint32_t gid[PF];
   auto take = [&]() -> int {
     if (got >= total) return 0;
-    const int n = GRID && TILE == 32 ? next_apart(src, gid) : src.next(gid);
+    const int n = GRID && TILE == 32 && PF == 1 ? next_apart(src, gid) : src.next(gid);
     if constexpr (GRID) {
       if (got + n > lcount) {   // the footprint count and the tile test disagree
         if (threadIdx.x == 0) atomicOr(&w.hdr->status, kStInternal);
