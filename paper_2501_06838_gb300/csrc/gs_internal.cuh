@@ -15,6 +15,7 @@ enum : uint32_t { kStInvalid = 1u, kStCapacity = 2u, kStInternal = 4u, kStTimeou
 constexpr int kSetupChunk = 16;       // image descriptors per setup launch
 constexpr int kFootprintBlock = 256;  // Gaussians per footprint / emit block
 constexpr int kRecordF4 = 4;          // a record is 4 float4 = 64 B
+constexpr int kFarReach = 1 << 30;    // grid binning: a reach of this many HR px or more
 constexpr int kGbCells = 64;          // LR cells at most per block of the block Gaussian-warp adjoint
 
 // Per-image descriptor, copied into the workspace at the start of each call.
@@ -97,6 +98,7 @@ struct Ws {
   short4* win;                // [N] windows (x0, y0, x1, y1) for grid binning, in output rows (from
                               // row0; empty: never meets a tile)
   int4* ext;                  // [n_images] reach (DL, DR, DT, DB) of the windows past their LR cell, HR px
+                              // (at most kFarReach)
   uint32_t* tcount;           // [T] grid mode: per-row differences of the (tile, Gaussian)
                               // pairs per tile (a tile's count is the prefix along its row)
   int64_t n;                  // total Gaussians

@@ -348,11 +348,12 @@ __global__ void __launch_bounds__(kFootprintBlock, 6) k_preprocess(Ws w, const _
                        : make_short4(32767, 32767, -32768, -32768);
       if (live) {
         const float sj = s * (float)F.j, si = s * (float)F.i;
-        reach.x = max(0, (int)ceilf(sj - (float)x0) + 1);
-        reach.y = max(0, (int)ceilf((float)x1 - sj) + 1);
         const int margin = 1 + (D.row0 >> 20);
-        reach.z = max(0, (int)ceilf(si - (float)y0) + margin);
-        reach.w = max(0, (int)ceilf((float)y1 - si) + margin);
+        auto past = [](float d, int more) { return d < (float)kFarReach ? max(0, (int)ceilf(d) + more) : kFarReach; };
+        reach.x = past(sj - (float)x0, 1);
+        reach.y = past((float)x1 - sj, 1);
+        reach.z = past(si - (float)y0, margin);
+        reach.w = past((float)y1 - si, margin);
         rim = im;
       }
     }

@@ -248,9 +248,9 @@ __device__ __forceinline__ void candidate_box(const Ws& w, const ImageDesc* D, i
   const int4 e = w.ext[D - w.images];   // HR px
   const float r = __frcp_rn(D->scale);
   const int j0 = max(0, (int)ceilf((float)(X0 - e.y) * r));
-  const int j1 = min(D->lr_w - 1, (int)floorf((float)(X1 + e.x) * r));
+  const int j1 = e.x < kFarReach ? min(D->lr_w - 1, (int)floorf((float)(X1 + e.x) * r)) : D->lr_w - 1;
   const int i0 = max(0, (int)ceilf((float)(Y0 - e.w) * r));
-  const int i1 = min(D->lr_h - 1, (int)floorf((float)(Y1 + e.z) * r));
+  const int i1 = e.z < kFarReach ? min(D->lr_h - 1, (int)floorf((float)(Y1 + e.z) * r)) : D->lr_h - 1;
   c.win = reinterpret_cast<const uint2*>(w.win);
   c.rstride = (int64_t)D->lr_w * D->m;
   c.rb0 = D->g_base + ((int64_t)i0 * D->lr_w + j0) * D->m;

@@ -1,12 +1,11 @@
 """Gaussians whose window lies far from their LR cell (a huge scale, offsets that
-bring the centres back to the origin): grid binning either finds them or says
-that its lists are incomplete; it never returns a wrong image with a clean
-status."""
+bring the centres back to the origin), 2^31 HR px and more: grid binning finds
+them all, and its lists hold what the footprint pass counted."""
 import numpy as np
 import pytest
 
 import gs_synthetic as S
-from _util import device_gaussians
+from _util import device_gaussians, normwise
 
 pytestmark = pytest.mark.gpu
 SORT, GRID = 1, 2
@@ -29,17 +28,16 @@ def _scene(scale, lr_w):
 @pytest.mark.parametrize("scale,lr_w", [(1e6, 40), (1.5e8, 14), (1e9, 5), (1e12, 70)])
 @pytest.mark.parametrize("tile,batch,raster", [(8, 0, TILE), (8, 64, TILE), (16, 0, TILE), (16, 64, TILE),
                                                (16, 0, PAIR), (32, 0, TILE)])
-def test_far_cells_found_or_flagged(scale, lr_w, tile, batch, raster):
+def test_far_cells(scale, lr_w, tile, batch, raster):
+    import torch
     import paper_2501_06838_gb300 as gs
     g, v = _scene(scale, lr_w)
-    dg = device_gaussians(g)
-    v.binning = SORT
-    want, _ = gs.render(dg, v, tile=tile, batch=batch, check=True)
-    v.binning, v.raster = GRID, raster
-    got, ws = gs.render(dg, v, tile=tile, batch=batch)
-    try:
-        gs.sync_status(ws)
-    except gs.GsError as e:
-        assert e.status == 6   # GS_ERR_INTERNAL: the lists are not the footprint count's
-        return
-    assert np.array_equal(got.cpu().numpy(), want.cpu().numpy())
+    dg, imgs, grads = device_gaussians(g), [], []
+    go = torch.from_numpy(S.grad_out(65, v.out_h, v.out_w)).cuda()
+    for v.binning, v.raster in ((SORT, TILE), (GRID, raster)):
+        out, ws = gs.render(dg, v, tile=tile, batch=batch, check=True)
+        imgs.append(out.cpu().numpy())
+        grads.append(gs.render_bwd(dg, v, go, ws, tile=tile, batch=batch, check=True).cpu().double().numpy())
+    assert imgs[0].any() and np.array_equal(imgs[0], imgs[1])
+    # the same lists: sums of the same terms, in any order of a tile's parts
+    assert np.all(normwise(grads[1], grads[0], axis=0) < 1e-5)
