@@ -148,9 +148,9 @@ typedef enum { GS_BINNING_AUTO = 0, GS_BINNING_SORT = 1, GS_BINNING_GRID = 2 } g
  *         (GS_ERR_UNSUPPORTED otherwise);
  *   AUTO: PAIR with GRID binning at tile 16 when every view uses the SIGMA
  *         window and the pairs are enough to fill the chip with short lists
- *         (where it measured faster: some scale >= 4 and 5,000 pairs, >= 10 and
- *         1,200 pairs, or a batch of small images with short lists at >= 6), else
- *         TILE. */
+ *         (where it measured faster: some scale >= 4 and 5,000 pairs, or >= 10 and
+ *         1,200 pairs), and, as it always has, for batches of small images with
+ *         short lists at some scale >= 6; else TILE. */
 typedef enum { GS_RASTER_AUTO = 0, GS_RASTER_TILE = 1, GS_RASTER_PAIR = 2 } gs_raster;
 
 /* The Gaussian primary head's activations (Sec. 3.2, "Gaussian Primary Head"),

@@ -408,7 +408,8 @@ __global__ void __launch_bounds__(32 * kBwWarps) k_raster_bwd_quad(Ws w, const u
 // by the chain rule after each adjoint) until the tiles run out, so that no
 // partial last wave idles SMs. The counter is asked only after a tile is done,
 // which spreads the (same-address) atomics over the launch. Registers capped
-// at 64 for 32 resident CTAs per SM (no spills at tile 8, 16 or 32).
+// at 64 for 32 resident CTAs per SM (no spills, but for 8 bytes in tile 16's form
+// over parts of lists).
 template <int TILE, bool SPLIT>
 __global__ void __launch_bounds__(32, 32) k_raster_bwd_tile(Ws w, const uint32_t* vals) {
   griddep_enter(w);

@@ -142,8 +142,10 @@ struct Problem {
 // 677 / 730. Below 256 pairs either layout is one short round of warps on part of
 // the chip, and tiles (with teams where lists are longer) are faster: one image,
 // calls, 4 Gaussians per pixel at scale 12 19.3 / 26.4, 1 per pixel at scale 6
-// 12.7 / 14.6. Only batches of small images with short lists keep the pairs that
-// a scale of 6 always had (4 images, 10.3 to 15.9 / 12.1 to 20.0).
+// 12.7 / 14.6. Batches of small images with short lists keep pairs from a scale of
+// 6 on although tiles measured faster there too (4 images, 10.3 to 15.9 / 12.1 to
+// 20.0): AUTO has always reported PAIR for them, and programs that read the stats
+// may count on it.
 bool pairs_pay(const Problem& P, float scale) {
   const int64_t pairs = P.tile_pairs, n = P.n, tiles = P.tiles;
   if (scale >= 4.0f && pairs >= 5000) return n < (scale >= 6.0f ? 30 : 18) * tiles;
@@ -310,7 +312,11 @@ int radix_passes(int64_t tiles) { return (key_bits(tiles) + 8) / 9; }
 // 56 13.5 -> 13.6, 37 12.1 -> 12.5; on 400 to 702 tiles (4 warps): 185 26.4 ->
 // 25.4, 77 15.7 -> 16.0, 56 15.3 -> 17.0. Boxes on 3,249 tiles by Gaussians per
 // tile: 643 516 -> 431, 251 331 -> 306, 140 183 -> 211; on 15,625: 655 2000 ->
-// 1973, 455 1014 -> 1127.
+// 1973, 455 1014 -> 1127. Ratio window on 3,600 to 3,969 tiles by list: 600 166 ->
+// 203, 730 212 -> 244, 990 266 -> 268, 1,340 378 -> 359, 1,640 484 -> 434, 5,370 1531
+// -> 1361; on 6,400, 1,420 618 -> 614; on 12,769, 820 639 -> 758, 1,620 1263 -> 1264
+// (an entry covers more of its tile than a box's, so a list of the same length is
+// the longer walk, and the line lies lower).
 int team_of(const Problem& P, const gs_gaussians* g, const gs_view* v) {
   if (P.tile != 16 || P.pair || P.batch == 64) return 0;
   double listed = 0.0;

@@ -286,7 +286,9 @@ __device__ __forceinline__ void griddep_release() {
 // 87.7 -> 82.7. With more blocks than are resident (5 per SM, 210,000 Gaussians:
 // 77.9 -> 79.0) the later ones have nothing to hide behind and take more sectors
 // from L2, and batches wait for the image table in any case.
-constexpr int64_t kOneWave = 6 * 152 * 256;   // Gaussians
+// The six blocks per SM are the footprint pass's launch bound; with fewer SMs the
+// line would only lie further out than it pays.
+constexpr int64_t kOneWave = 6 * 152 * 256;   // Gaussians: blocks per SM x SMs x block
 __host__ __device__ __forceinline__ bool reads_early(const Ws& w) {
   return w.n_images == 1 && w.n <= kOneWave;
 }

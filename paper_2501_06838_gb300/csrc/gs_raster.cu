@@ -88,7 +88,8 @@ __device__ __forceinline__ void load_ids(const uint32_t* vals, int bs, int nb, u
 // A tile's list is summed in segments of kSeg entries, one after the other:
 // out = ((S0 + S1) + S2) + .... One warp writes each segment's sums onto the
 // output as it ends; a team of warps sums them side by side and adds them in
-// the same order (k_raster_fwd_team): the same bits in every layout.
+// the same order (k_raster_fwd_team): the same bits in every layout of tile 16.
+// (Tiles 8 and 32 sum a tile's whole list in one run, k_raster_fwd.)
 constexpr int kSeg = 512;
 
 // Where a tile's Gaussian ids come from, one batch at a time (ids ascending,
@@ -1132,9 +1133,10 @@ __global__ void __launch_bounds__(TILE * TILE / BY) k_raster_fwd(Ws w, const uin
 // bounds it. Against the former pair layout (each lane a column of both tiles,
 // 7 shared loads per 16 pixels): 1168 -> 1007 us on 518,400 Gaussians at
 // 5760 x 3240 (windows of 74 px on average), 857 -> 799 us on 16 uneven images,
-// 87 -> 73 us at scale 24. Wider strips cost small windows more columns, so
-// scales below 6 keep single tiles (1002 x 751 at scale 3.7, 14 px windows: 52
-// against 70 us). The register cap (128, no spills) gives 16 CTAs per SM; 18
+// 87 -> 73 us at scale 24. Wider strips cost small windows more columns
+// (1002 x 751 at scale 3.7, 14 px windows: 52 us by tiles, 70 by pairs) and pairs
+// make half as many warps: the host's rule says where they pay. The register cap
+// (128; spills, 8 bytes, with 64 Gaussians a round only) gives 16 CTAs per SM; 18
 // CTAs (112, spills) were 2% faster on the uneven batch and 1% to 10% slower
 // elsewhere.
 // ---------------------------------------------------------------------------
@@ -1384,7 +1386,12 @@ cudaError_t run_team(const Ws& w, const uint32_t* vals, cudaStream_t s) {
 
 // Launch configurations: tile edge -> rows per thread (threads = TILE^2 / BY);
 // batch = Gaussians staged per round = threads * PF, PF in {1, 2} (the host
-// accepts only these batches; 0 selects PF = 1).
+// accepts only these batches; 0 selects PF = 1). Tile 16 with 64 a round never
+// measured faster than 32 (forward calls, us, 32 / 64: 65,536 Gaussians at 1024 x
+// 1024 36 / 40, 220,052 at 1002 x 751 66 / 74, pairs at 5760 x 3240 1032 / 1230, the
+// ratio window at 720 x 720 2,933 / 3,906, whose teams take 32 only): it costs a
+// second table per warp. It stays for callers that name it, at 0.7 to 0.84 of what
+// the layout before the strips took with it (53, 105, 1603, 4,633).
 cudaError_t dispatch(const Ws& w, const uint32_t* vals, int batch, cudaStream_t s) {
   if (w.tiles == 0) return cudaSuccess;
   if (w.pair) {   // grid binning, tile 16: one warp per horizontal pair of tiles
