@@ -59,15 +59,15 @@ PAIR_CYCLES = {"raster_fwd": 6.5, "raster_bwd": 12.0, "raster_bwd_gw": 12.0}
 # source they were taken on: reported as null once that source file changes.
 TRAFFIC = {
     ("c2", "raster_bwd"): ("gs_adjoint_tile.cu",
-                           "73b41edd332ba9febab557472d55993aae9f872c51f833f52eabf6470f7129c8",
+                           "1057ba7cb7fd4ad0a74393be749080447af730a42808d0fcd8f423bea036a214",
                            21310976 + 0, "profiles/raster_bwd_c2_1024x1024.md"),
     ("c4x12-bf16", "raster_bwd"): ("gs_adjoint_tile.cu",
-                                   "73b41edd332ba9febab557472d55993aae9f872c51f833f52eabf6470f7129c8",
-                                   350088704 + 21108480,
+                                   "1057ba7cb7fd4ad0a74393be749080447af730a42808d0fcd8f423bea036a214",
+                                   350338560 + 21283072,
                                    "profiles/raster_bwd_c4x12_bf16_5760x3240.md"),
     ("c4x12-bf16", "raster_fwd"): ("gs_raster.cu",
-                                   "7d54d7101ecc6906751ede1a417846269f59e94b1bca9ef0d6d2255aa3bf690d",
-                                   37683968 + 227410432,
+                                   "b52508e82acb9ad0018d8cb0b05f4ba17d8b2f84f9932244714cc93080c1b87e",
+                                   37671936 + 227354368,
                                    "profiles/raster_fwd_c4x12_bf16_5760x3240.md"),
 }
 

@@ -234,13 +234,13 @@ __device__ __forceinline__ void cp_async16z(void* smem, const void* gmem, int sr
 
 // Block form, for Gaussians on a reference grid (m > 0): one CTA per block of
 // gb_x x gb_y LR cells of an image (the host picks the shape: gblock_shape).
-// The CTA first forms the union box of its Gaussians' windows and, when the box fits kGbFloats, copies the
-// upstream gradient over it into shared memory once (three planes, the first
-// column even and the width even); its warps then walk their Gaussians (the
-// k-th of the block goes to warp k % kGbWarps) exactly as the one-warp form
-// does, reading the gradient from shared memory instead of L1/L2. A block
-// whose box does not fit walks the gradient in global memory. Each Gaussian's
-// sums keep the one-warp form's order, so the moments are the same bits.
+// The CTA first forms the union box of its Gaussians' windows and, when the box
+// fits kGbFloats, copies the upstream gradient over it into shared memory once
+// (three planes, the first column even and the width even); its warps then walk
+// their Gaussians (the k-th of the block goes to warp k % kGbWarps) exactly as
+// the one-warp form does, reading the gradient from shared memory instead of
+// L1/L2. A block whose box does not fit walks the gradient in global memory. Each
+// Gaussian's sums keep the one-warp form's order, so the moments are the same bits.
 constexpr int kGbWarps = 8;
 constexpr int kGbFloats = 24 * 1024;   // 96 KB of staged gradient at most
 
