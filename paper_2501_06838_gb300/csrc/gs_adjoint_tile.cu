@@ -446,12 +446,16 @@ namespace {
 // which the pair capacity bounds (sized by a count, it is the mean), or into as
 // many as make `spare` CTAs in all: those are next to free, and shorten what one
 // long list among short ones takes. Adjoint, us, whole lists / cut so / a chip's
-// worth of parts: tile 16, 256 tiles, lists of 16 9.7 / 10.4 / 16.3, 62 19.2 / 12.7
-// / 18.7, 125 33.5 / 16.4 / 21.7; 1,024 tiles, 16 12.1 / 12.1 / 21.2, 64 27.6 / 25.3
-// / 26.5; 2,025 tiles, 16 15.6 / 15.6 / 24.7, 64 42.8 / 30.1 / 31.3; quadrants, 256
-// tiles, 63 9.4 / 9.4 / 10.3, 250 16.0 / 14.8 / 15.6. With half the Gaussians in a
-// 25th of the tiles: tile 16, 64 tiles, mean 14 26.1 / 9.6 / 10.4, 256 tiles, 62 132
-// / 41 / 19; quadrants, 256 tiles, 62 27.8 / 12.7 / 10.7.
+// worth of parts. Tile 16 (16 entries, 512 CTAs), 256 tiles, lists of 16 9.7 / 10.4
+// / 16.3, 62 19.2 / 12.7 / 18.7, 125 33.5 / 16.4 / 21.7; 1,024 tiles, 16 12.1 / 12.1
+// / 21.2, 64 27.6 / 25.3 / 26.5; 2,025 tiles, 16 15.6 / 15.6 / 24.7. Quadrants (16,
+// 512), 256 tiles, 63 9.4 / 9.4 / 10.3. Tile 8 (24, 2,048), 1,024 tiles, 7 10.0 / 9.8
+// / 14.1, 44 10.6 / 10.5 / 16.1, 176 23.9 / 21 / 22.7. Tile 32 (6, 512), 400 tiles, 8
+// 23.0 / 23.0 / 41.0, 49 56.5 / 48 / 48.9. With half the Gaussians in a 25th of the
+// tiles: tile 16, 64 tiles, mean 14 26.1 / 9.6 / 10.4, 256 tiles, 62 132 / 41 / 19;
+// quadrants, 256 tiles, 62 27.8 / 12.7 / 10.7. Over 449 such scenes and reference
+// grids, forward and adjoint together, at most 10% slower than whole lists
+// anywhere, where a chip's worth took up to 33% more.
 int32_t list_parts(const Ws& w, int64_t full, int64_t entries, int64_t spare) {
   const int64_t tiles = w.tiles;
   if (2 * tiles > full) return 1;
@@ -475,12 +479,11 @@ BwdKernel tile_kernel(int tile, bool split) {
 }  // namespace
 
 int32_t raster_bwd_parts(const Ws& w, bool quadrants) {
-  // a chunk of a quadrant CTA is four warps', one of an 8 x 8 tile a quarter of the work
   if (quadrants)
     return list_parts(w, resident_grid((const void*)k_raster_bwd_quad<false>, 32 * kBwWarps, INT32_MAX),
-                      64, 1024);
+                      16, 512);
   return list_parts(w, resident_grid((const void*)tile_kernel(w.tile, false), 32, INT32_MAX),
-                    w.tile == 8 ? 64 : 16, 512);
+                    w.tile == 8 ? 24 : w.tile == 32 ? 6 : 16, w.tile == 8 ? 2048 : 512);
 }
 
 cudaError_t launch_raster_bwd_tile(const Ws& ws, const uint32_t* lists, bool quadrants,

@@ -35,8 +35,9 @@ def test_split_lists(n, mode, tile):
     assert np.all(err < 1e-5), err
 
 
-@pytest.mark.parametrize("mode,tile,edge,longest,whole", [(TILE, 8, 30, 95, 1), (TILE, 16, 30, 23, 1),
-                                                          (TILE, 32, 30, 23, 1), (QUADRANT, 16, 20, 159, 2)])
+@pytest.mark.parametrize("mode,tile,edge,longest,whole", [(TILE, 8, 46, 35, 1), (TILE, 8, 30, 59, 2),
+                                                          (TILE, 16, 30, 23, 1), (TILE, 32, 30, 8, 1),
+                                                          (QUADRANT, 16, 20, 23, 1)])
 def test_short_lists_stay_whole(mode, tile, edge, longest, whole):
     """A part costs a CTA, so short lists are not cut for the chip's sake, or only
     as far as the CTAs are next to free; a larger workspace (whose capacity no
