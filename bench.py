@@ -59,15 +59,15 @@ PAIR_CYCLES = {"raster_fwd": 6.5, "raster_bwd": 12.0, "raster_bwd_gw": 12.0}
 # source they were taken on: reported as null once that source file changes.
 TRAFFIC = {
     ("c2", "raster_bwd"): ("gs_adjoint_tile.cu",
-                           "1057ba7cb7fd4ad0a74393be749080447af730a42808d0fcd8f423bea036a214",
-                           21310976 + 0, "profiles/raster_bwd_c2_1024x1024.md"),
+                           "d839bd08224b9ebbb6e28832ee8ebe81620493a22fc2b3c0bda8d20c743c57ed",
+                           21310720 + 0, "profiles/raster_bwd_c2_1024x1024.md"),
     ("c4x12-bf16", "raster_bwd"): ("gs_adjoint_tile.cu",
-                                   "1057ba7cb7fd4ad0a74393be749080447af730a42808d0fcd8f423bea036a214",
-                                   350338560 + 21283072,
+                                   "d839bd08224b9ebbb6e28832ee8ebe81620493a22fc2b3c0bda8d20c743c57ed",
+                                   350122752 + 21211648,
                                    "profiles/raster_bwd_c4x12_bf16_5760x3240.md"),
     ("c4x12-bf16", "raster_fwd"): ("gs_raster.cu",
                                    "b52508e82acb9ad0018d8cb0b05f4ba17d8b2f84f9932244714cc93080c1b87e",
-                                   37671936 + 227354368,
+                                   37702400 + 226898176,
                                    "profiles/raster_fwd_c4x12_bf16_5760x3240.md"),
 }
 
